@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(FTC_THREADS, FtcCfg<DUAL>::CTAS)
   pdl_entry();
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---- TMA producer ---------------------------------------------------------------
       mbar_expect_tx(&q_full, C::Q_B);
       tma_load_3d(sQ, &tmQ, &q_full, 0, row0 + qt * TQ, 0);
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(FTC_THREADS, FtcCfg<DUAL>::CTAS)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---- MMA issuer -------------------------------------------------------------------
       const uint32_t idS = idesc_bf16(TQ, TK);
       const uint32_t idO = idesc_bf16(TQ, HD) | (1u << 16);   // B (V) read MN-major
@@ -707,7 +707,7 @@ __global__ void __launch_bounds__(BW_THREADS, KvCfg<DUAL>::CTAS)
   pdl_entry();
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---- TMA producer ---------------------------------------------------------------
       mbar_expect_tx(&res_full, C::NRES * ROWS128_B);
       tma_load_3d(sRes, &tmK, &res_full, 0, row0 + key0, 0);
@@ -741,7 +741,7 @@ __global__ void __launch_bounds__(BW_THREADS, KvCfg<DUAL>::CTAS)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---- MMA issuer -------------------------------------------------------------------
       const uint32_t idS = idesc_bf16(128, BT_Q);
       const uint32_t idA = idesc_bf16(128, HD) | (1u << 16);   // B (Q, dO) read MN-major
@@ -1032,7 +1032,7 @@ __global__ void __launch_bounds__(BW_THREADS, QCfg<DUAL>::CTAS)
   pdl_entry();
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---- TMA producer ---------------------------------------------------------------
       mbar_expect_tx(&res_full, C::NRES * ROWS128_B);
       tma_load_3d(sRes, &tmQ, &res_full, 0, row0 + q0, 0);
@@ -1061,7 +1061,7 @@ __global__ void __launch_bounds__(BW_THREADS, QCfg<DUAL>::CTAS)
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---- MMA issuer -------------------------------------------------------------------
       const uint32_t idS = idesc_bf16(128, BT_Q);
       const uint32_t idA = idesc_bf16(128, HD) | (1u << 16);   // B (K) read MN-major

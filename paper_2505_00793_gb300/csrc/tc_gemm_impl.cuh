@@ -96,6 +96,20 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// True in one lane of a converged warp.  The roles that issue TMA loads and MMAs branch on
+// this rather than on lane == 0: the instructions take their operands from uniform
+// registers, and only elect.sync tells the compiler that a single lane is active, which
+// spares it a loop over lanes around every one of them.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r));
+  return r != 0;
+}
+
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
 }
@@ -743,6 +757,88 @@ __device__ __forceinline__ void mma_commit_pair_addr(uint32_t addr) {
       : "memory");
 }
 
+__device__ __forceinline__ void mbar_expect_tx_addr(uint32_t addr, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(addr), "r"(bytes)
+               : "memory");
+}
+
+// A TMA load of a 3-D box into shared memory (PAIR: the cta_group::2 form, whose barrier may
+// be the peer CTA's), on precomputed addresses.
+template <bool PAIR>
+__device__ __forceinline__ void tma_load_at(uint32_t dst, const CUtensorMap* map, uint32_t bar,
+                                            int x, int y, int z) {
+  if constexpr (PAIR)
+    asm volatile(
+        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar)
+        : "memory");
+  else
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar)
+        : "memory");
+}
+
+// The TMA producer's position in the stage ring: the stage's barrier and data addresses and
+// its phase, advanced by additions.  One thread issues every load, so its instructions per
+// K block bound the pipeline of tiles whose MMAs are short: with a division by the stage
+// count and rebuilt addresses it took about 1000 clocks per K block, twice the MMAs of a
+// 256 x 256 pair tile.
+struct LoadRing {
+  uint32_t full0, empty0, base, full, empty, dst, ph;
+  int s, stages, stage_bytes;
+  __device__ __forceinline__ LoadRing(uint32_t f, uint32_t e, uint32_t b, int n, int bytes)
+      : full0(f), empty0(e), base(b), full(f), empty(e), dst(b), ph(0), s(0), stages(n),
+        stage_bytes(bytes) {}
+  __device__ __forceinline__ void next() {
+    if (++s == stages) {
+      s = 0;
+      ph ^= 1u;
+      full = full0; empty = empty0; dst = base;
+    } else {
+      full += 8u; empty += 8u;
+      dst += static_cast<uint32_t>(stage_bytes);
+    }
+  }
+};
+
+// The loads of one K block at k: 128 rows of A from m0, BROWS rows of B from n0.
+template <int BROWS, int KA, bool PAIR>
+__device__ __forceinline__ void load_block(const LoadRing& R, const TcParams& p,
+                                           const CUtensorMap* A0, const CUtensorMap* A1,
+                                           const CUtensorMap* B0, const CUtensorMap* B1, int m0,
+                                           int n0, int k, int bz) {
+  constexpr uint32_t A_ATOM = BM * BK * 2, B_ATOM = BROWS * BK * 2;
+#pragma unroll
+  for (int a = 0; a < KA; ++a) {
+    const int ka = k + a * BK;
+    const uint32_t a0 = R.dst + p.a0_off, a1 = R.dst + p.a1_off;
+    const uint32_t b0 = R.dst + p.b0_off, b1 = R.dst + p.b1_off;
+    if (p.a_mn) {   // MN-major: boxes of 64 rows x 64 K at (row, k)
+#pragma unroll
+      for (int j = 0; j < BM / 64; ++j) {
+        if (p.a0_off >= 0) tma_load_at<PAIR>(a0 + j * MN_BOX, A0, R.full, m0 + 64 * j, ka, bz);
+        if (p.a1_off >= 0) tma_load_at<PAIR>(a1 + j * MN_BOX, A1, R.full, m0 + 64 * j, ka, bz);
+      }
+    } else {
+      if (p.a0_off >= 0) tma_load_at<PAIR>(a0 + a * A_ATOM, A0, R.full, ka, m0, bz);
+      if (p.a1_off >= 0) tma_load_at<PAIR>(a1 + a * A_ATOM, A1, R.full, ka, m0, bz);
+    }
+    if (p.b_mn) {
+#pragma unroll
+      for (int j = 0; j < BROWS / 64; ++j) {
+        if (p.b0_off >= 0) tma_load_at<PAIR>(b0 + j * MN_BOX, B0, R.full, n0 + 64 * j, ka, bz);
+        if (p.b1_off >= 0) tma_load_at<PAIR>(b1 + j * MN_BOX, B1, R.full, n0 + 64 * j, ka, bz);
+      }
+    } else {
+      if (p.b0_off >= 0) tma_load_at<PAIR>(b0 + a * B_ATOM, B0, R.full, ka, n0, bz);
+      if (p.b1_off >= 0) tma_load_at<PAIR>(b1 + a * B_ATOM, B1, R.full, ka, n0, bz);
+    }
+  }
+}
+
 // Shared-memory descriptors of one operand for stage 0 of the ring.  The descriptor's
 // address field holds (address & 0x3FFFF) >> 4 in its low 14 bits, and every stage, K atom
 // and K slice lies inside the CTA's shared memory, so moving a descriptor by a byte offset
@@ -940,47 +1036,21 @@ __global__ void __launch_bounds__(THREADS, 1)
   pdl_entry();
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---- TMA producer: KA swizzle atoms per operand per stage -------------------------
-      const int stages = p.stages, stage_bytes = p.stage_bytes, tx_bytes = p.tx_bytes;
-      const int a0_off = p.a0_off, a1_off = p.a1_off, b0_off = p.b0_off, b1_off = p.b1_off;
-      int* const status = p.status;
+      LoadRing R(smem_u32(full_bar), smem_u32(empty_bar), smem_u32(smem), p.stages, p.stage_bytes);
       int issued = 0;
       for (int i = 0; i < nk; ++i, ++issued) {
-        const int s = i % stages;
-        const uint32_t ph = (i / stages) & 1;
-        if (!mbar_wait(&empty_bar[s], ph ^ 1, status, DRAIN_NS)) break;
-        uint8_t* st = smem + s * stage_bytes;
-        mbar_expect_tx(&full_bar[s], tx_bytes);
-        const int k = (kb0 + i) * SK;
-#pragma unroll
-        for (int a = 0; a < KA; ++a) {
-          const int ka = k + a * BK;
-          if (p.a_mn) {   // MN-major: boxes of 64 rows x 64 K at (row, k)
-            for (int j = 0; j < BM / 64; ++j) {
-              if (a0_off >= 0) tma_load_3d(st + a0_off + j * MN_BOX, &tmA0, &full_bar[s], m0 + 64 * j, ka, bz);
-              if (a1_off >= 0) tma_load_3d(st + a1_off + j * MN_BOX, &tmA1, &full_bar[s], m0 + 64 * j, ka, bz);
-            }
-          } else {
-            if (a0_off >= 0) tma_load_3d(st + a0_off + a * A_ATOM, &tmA0, &full_bar[s], ka, m0, bz);
-            if (a1_off >= 0) tma_load_3d(st + a1_off + a * A_ATOM, &tmA1, &full_bar[s], ka, m0, bz);
-          }
-          if (p.b_mn) {
-            for (int j = 0; j < BN / 64; ++j) {
-              if (b0_off >= 0) tma_load_3d(st + b0_off + j * MN_BOX, &tmB0, &full_bar[s], n0 + 64 * j, ka, bz);
-              if (b1_off >= 0) tma_load_3d(st + b1_off + j * MN_BOX, &tmB1, &full_bar[s], n0 + 64 * j, ka, bz);
-            }
-          } else {
-            if (b0_off >= 0) tma_load_3d(st + b0_off + a * B_ATOM, &tmB0, &full_bar[s], ka, n0, bz);
-            if (b1_off >= 0) tma_load_3d(st + b1_off + a * B_ATOM, &tmB1, &full_bar[s], ka, n0, bz);
-          }
-        }
+        if (!mbar_wait_addr(R.empty, R.ph ^ 1u, p.status, DRAIN_NS)) break;
+        mbar_expect_tx_addr(R.full, static_cast<uint32_t>(p.tx_bytes));
+        load_block<BN, KA, false>(R, p, &tmA0, &tmA1, &tmB0, &tmB1, m0, n0, (kb0 + i) * SK, bz);
+        R.next();
       }
-      drain_loads(full_bar, issued, stages, status);
+      drain_loads(full_bar, issued, p.stages, p.status);
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0 && nk > 0) {
+    if (nk > 0 && elect_one()) {
       // ---- MMA issuer (single thread) -----------------------------------------------
       MmaLoop L;
       L.nk = nk; L.stages = p.stages; L.stage_bytes = p.stage_bytes;
@@ -1399,47 +1469,24 @@ __global__ void __launch_bounds__(THREADS2, 1)
   pdl_entry();
 
   if (warp == 0) {
-    if (lane == 0) {
-      const int stages = p.stages, stage_bytes = p.stage_bytes;
-      const int a0_off = p.a0_off, a1_off = p.a1_off, b0_off = p.b0_off, b1_off = p.b1_off;
-      int* const status = p.status;
-      const uint32_t full0 = dsmem_addr(smem_u32(&full_bar[0]), 0);   // even CTA's barriers
+    if (elect_one()) {
+      LoadRing R(dsmem_addr(smem_u32(full_bar), 0), smem_u32(empty_bar), smem_u32(smem), p.stages,
+                 p.stage_bytes);   // full: the even CTA's barriers
       const int nb0 = n0 + static_cast<int>(rank) * BH;
       int issued = 0;
       for (int i = 0; i < nk; ++i, ++issued) {
-        const int s = i % stages;
-        const uint32_t ph = (i / stages) & 1;
-        if (!mbar_wait(&empty_bar[s], ph ^ 1, status, DRAIN_NS)) break;
-        if (rank == 0) mbar_expect_tx(&full_bar[s], 2 * stage_bytes);
-        const uint32_t bar = full0 + static_cast<uint32_t>(s) * 8u;
-        uint8_t* st = smem + s * stage_bytes;
-        const int k = i * BK;
-        if (p.a_mn) {
-          for (int j = 0; j < BM / 64; ++j) {
-            if (a0_off >= 0) tma_load_3d_pair(st + a0_off + j * MN_BOX, &tmA0, bar, m0 + 64 * j, k, bz);
-            if (a1_off >= 0) tma_load_3d_pair(st + a1_off + j * MN_BOX, &tmA1, bar, m0 + 64 * j, k, bz);
-          }
-        } else {
-          if (a0_off >= 0) tma_load_3d_pair(st + a0_off, &tmA0, bar, k, m0, bz);
-          if (a1_off >= 0) tma_load_3d_pair(st + a1_off, &tmA1, bar, k, m0, bz);
-        }
-        if (p.b_mn) {
-          for (int j = 0; j < BH / 64; ++j) {
-            if (b0_off >= 0) tma_load_3d_pair(st + b0_off + j * MN_BOX, &tmB0, bar, nb0 + 64 * j, k, bz);
-            if (b1_off >= 0) tma_load_3d_pair(st + b1_off + j * MN_BOX, &tmB1, bar, nb0 + 64 * j, k, bz);
-          }
-        } else {
-          if (b0_off >= 0) tma_load_3d_pair(st + b0_off, &tmB0, bar, k, nb0, bz);
-          if (b1_off >= 0) tma_load_3d_pair(st + b1_off, &tmB1, bar, k, nb0, bz);
-        }
+        if (!mbar_wait_addr(R.empty, R.ph ^ 1u, p.status, DRAIN_NS)) break;
+        if (rank == 0) mbar_expect_tx(&full_bar[R.s], 2 * p.stage_bytes);
+        load_block<BH, 1, true>(R, p, &tmA0, &tmA1, &tmB0, &tmB1, m0, nb0, i * BK, bz);
+        R.next();
       }
       // both CTAs' loads signal the even CTA's full barriers; the odd CTA's producer sees
       // the same commits and stops at the same stage, and waits at the final cluster barrier
-      if (rank == 0) drain_loads(full_bar, issued, stages, status);
+      if (rank == 0) drain_loads(full_bar, issued, p.stages, p.status);
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (rank == 0 && lane == 0) {
+    if (rank == 0 && elect_one()) {
       MmaLoop L;
       L.nk = nk; L.stages = p.stages; L.stage_bytes = p.stage_bytes;
       L.a0_off = p.a0_off; L.a1_off = p.a1_off; L.b0_off = p.b0_off; L.b1_off = p.b1_off;

@@ -301,13 +301,11 @@ __global__ void __launch_bounds__(threads_p<MODE>(), 1)
   };
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       // ---- TMA producer: this CTA's 128 rows of A and BN/2 rows of B per stage ------------
-      const int stages = p.stages, stage_bytes = p.stage_bytes;
-      const int a0_off = p.a0_off, a1_off = p.a1_off, b0_off = p.b0_off, b1_off = p.b1_off;
-      int* const status = p.status;
-      const uint32_t full0 = dsmem_addr(smem_u32(&full_bar[0]), 0);   // even CTA's barriers
-      int g = 0;   // K blocks issued so far (ring position)
+      LoadRing R(dsmem_addr(smem_u32(full_bar), 0), smem_u32(empty_bar), smem_u32(smem), p.stages,
+                 p.stage_bytes);   // full: the even CTA's barriers
+      int g = 0;   // K blocks issued so far
       bool live = true;
       for (int t = pair; t < pp.ntiles && live; t += npairs) {
         int bz, mp, tn;
@@ -315,38 +313,17 @@ __global__ void __launch_bounds__(threads_p<MODE>(), 1)
         const int m0 = mp * (2 * BM) + static_cast<int>(rank) * BM;
         const int nb0 = tn * BN + static_cast<int>(rank) * BH;
         for (int i = 0; i < nk; ++i, ++g) {
-          const int s = g % stages;
-          const uint32_t ph = (g / stages) & 1;
-          if (!mbar_wait(&empty_bar[s], ph ^ 1, status, DRAIN_NS)) { live = false; break; }
-          if (rank == 0) mbar_expect_tx(&full_bar[s], 2 * stage_bytes);
-          const uint32_t bar = full0 + static_cast<uint32_t>(s) * 8u;
-          uint8_t* st = smem + s * stage_bytes;
-          const int k = i * BK;
-          if (p.a_mn) {
-            for (int j = 0; j < BM / 64; ++j) {
-              if (a0_off >= 0) tma_load_3d_pair(st + a0_off + j * MN_BOX, &tmA0, bar, m0 + 64 * j, k, bz);
-              if (a1_off >= 0) tma_load_3d_pair(st + a1_off + j * MN_BOX, &tmA1, bar, m0 + 64 * j, k, bz);
-            }
-          } else {
-            if (a0_off >= 0) tma_load_3d_pair(st + a0_off, &tmA0, bar, k, m0, bz);
-            if (a1_off >= 0) tma_load_3d_pair(st + a1_off, &tmA1, bar, k, m0, bz);
-          }
-          if (p.b_mn) {
-            for (int j = 0; j < BH / 64; ++j) {
-              if (b0_off >= 0) tma_load_3d_pair(st + b0_off + j * MN_BOX, &tmB0, bar, nb0 + 64 * j, k, bz);
-              if (b1_off >= 0) tma_load_3d_pair(st + b1_off + j * MN_BOX, &tmB1, bar, nb0 + 64 * j, k, bz);
-            }
-          } else {
-            if (b0_off >= 0) tma_load_3d_pair(st + b0_off, &tmB0, bar, k, nb0, bz);
-            if (b1_off >= 0) tma_load_3d_pair(st + b1_off, &tmB1, bar, k, nb0, bz);
-          }
+          if (!mbar_wait_addr(R.empty, R.ph ^ 1u, p.status, DRAIN_NS)) { live = false; break; }
+          if (rank == 0) mbar_expect_tx(&full_bar[R.s], 2 * p.stage_bytes);
+          load_block<BH, 1, true>(R, p, &tmA0, &tmA1, &tmB0, &tmB1, m0, nb0, i * BK, bz);
+          R.next();
         }
       }
-      if (rank == 0) drain_loads(full_bar, g, stages, status);
+      if (rank == 0) drain_loads(full_bar, g, p.stages, p.status);
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (rank == 0 && lane == 0) {
+    if (rank == 0 && elect_one()) {
       // ---- MMA issuer (single thread of the even CTA) ------------------------------------
       MmaLoop L;
       L.nk = nk; L.stages = p.stages; L.stage_bytes = p.stage_bytes;
