@@ -16,9 +16,9 @@
 // (64-row boxes), so no operand is ever stored transposed. Each product term (MMA) rotates over
 // up to four TMEM accumulator blocks so that dependent MMAs do not serialise. CTA-pair tiles
 // (cta_group::2, 256 rows) serve GEMMs whose pair grid fills the GPU. GEMMs with few output
-// tiles split K across a thread-block cluster of S CTAs: the partial accumulators meet in
-// distributed shared memory, and each CTA reduces 128/S rows in a fixed order, so results are
-// deterministic. Every mbarrier wait is bounded; on expiry the CTA records DEV_TIMEOUT, stops
+// tiles split K across a thread-block cluster of S CTAs: each CTA bulk-copies its partial
+// rows to their owners' shared memory and adds the 128/S rows it owns in a fixed order, so
+// results are deterministic. Every mbarrier wait is bounded; on expiry the CTA records DEV_TIMEOUT, stops
 // issuing MMAs and drains the loads and MMAs it has issued before it releases its memory.
 #include "tc_gemm_impl.cuh"
 
