@@ -394,6 +394,7 @@ struct Exec {
   mf_status st = MF_OK;
   mf::LayerTable tab;
   bool ror_store = false;   // primal backward keeps every layer's dz (and da) for RoR
+  bool keep_d2 = false;     // primal forward leaves phi''(z) of the hidden layers for RoR
 
   // backward seed buffers of layer l (ping-pong, or the stored reverse graph)
   T* dz_buf(int l) const { return ror_store ? at<T>(p.o_SZ[l]) : at<T>(p.o_dZ[l & 1]); }
@@ -605,6 +606,7 @@ struct Exec {
         g.bias1 = h->md.has_bias ? u + h->boff[l] : nullptr;
       }
       if (l + 1 < h->L) {
+        if (keep_d2) { g.C1 = at<float>(p.o_Zd[l]); g.ldc1 = dout; }
         g.epi.mode = mf::EPI_ACT_FWD;
         g.epi.act = h->md.act;
         g.epi.A = at<T>(p.o_A[l + 1]);
@@ -655,7 +657,6 @@ struct Exec {
     const int L = h->L, l = L - 1, din = h->dims[l], dout = h->dims[L];
     mf::HeadArgs ha;
     ha.rows = rows; ha.D = din; ha.C = dout; ha.dual = dual;
-    ha.act = h->md.act;
     ha.A = at<T>(p.o_A[l]);
     ha.Ad = dual && l > 0 ? at<T>(p.o_Ad[l]) : nullptr;
     ha.lda = p.lda[l];
@@ -776,7 +777,9 @@ struct Exec {
                float* d_eta) {
     const int L = h->L, hb = h->md.has_bias ? 1 : 0;
     no_fuse = true;
+    keep_d2 = true;
     forward(rows, x, theta, nullptr, false);
+    keep_d2 = false;
     ror_store = true;
     loss(rows, false, y, eta_w, ex_w, nullptr, nullptr, nullptr);
     backward(rows, false, nullptr, grad);
@@ -797,7 +800,7 @@ struct Exec {
       g.bias0 = h->md.has_bias ? u + h->boff[l] : nullptr;
       gemm(g);
       if (l + 1 < L) {
-        mf::ror_fwd_elem<T>(h->md.act, at<float>(p.o_DZB), at<float>(p.o_Z[l]),
+        mf::ror_fwd_elem<T>(at<float>(p.o_DZB), at<float>(p.o_Z[l]), at<float>(p.o_Zd[l]),
                             at<float>(p.o_SA[l + 1]), rows, dout, at<T>(p.o_DAB[l]), p.lda[l + 1],
                             at<float>(p.o_ZP[l]), s);
         launched();
@@ -830,8 +833,8 @@ struct Exec {
     for (int l = L - 1; l >= 0; --l) {
       const int din = h->dims[l], dout = h->dims[l + 1];
       if (l + 1 < L) {
-        mf::ror_bwd_elem<T>(h->md.act, at<float>(p.o_ZP[l]), at<float>(p.o_AB), at<float>(p.o_Z[l]),
-                            rows, dout, at<T>(p.o_ZB), ld8(dout), s);
+        mf::ror_bwd_elem<T>(at<float>(p.o_ZP[l]), at<float>(p.o_AB), at<float>(p.o_Z[l]), rows,
+                            dout, at<T>(p.o_ZB), ld8(dout), s);
         launched();
       }
       // (H v)_{W_l, b_l} = [a_{l-1}^T; 1] zbar_l + [dabar_{l-1}^T; 0] dz_l

@@ -414,7 +414,7 @@ struct DecExec {
                              at<float>(p.x2d[l]), at<float>(p.r2[l]), at<float>(p.r2d[l]),
                              at<T>(p.h2[l]), at<T>(p.h2d[l]), d, s);
       launched();
-      // a = GELU(h2 W1) fused; z kept for the backward
+      // a = GELU(h2 W1) fused; its derivatives (in z1, z1') kept for the backward
       {
         GemmArgs g = lin(N, F, d, at<T>(p.h2[l]), at<T>(p.h2d[l]), d, W(Ly.W1[l]), Uw(Ly.W1[l]),
                          ld8(F), dual);

@@ -46,39 +46,53 @@ __device__ __forceinline__ void act_eval(int act, float z, float& f, float& d1, 
 
 // Per-element epilogue of a dual GEMM (shared by the tensor-core and SIMT kernels).
 //  EPI_STORE:   C0 = acc0 + bias0, C1 = acc1 + bias1.
-//  EPI_ACT_FWD: z = acc0 + bias0, z' = acc1 + bias1 -> C0 = z, C1 = z' (float32),
-//               a = phi(z), a' = phi'(z) z'  -> A, Ad (row-major).
-//  EPI_ACT_BWD: da = acc0, da' = acc1, z, z' read from Z, Zd ->
-//               dz = phi'(z) da, dz' = phi''(z) z' da + phi'(z) da'  -> A, Ad.
+//  EPI_ACT_FWD: z = acc0 + bias0, z' = acc1 + bias1 ->
+//               a = phi(z), a' = phi'(z) z'  -> A, Ad (row-major), and what the backward pass
+//               needs of z, in place of z itself: phi'(z) -> C0 and, where C1 is given,
+//               phi''(z) z' (dual) or phi''(z) (primal) -> C1, float32.  The activation is
+//               evaluated once per element and pass instead of again in the backward.
+//  EPI_ACT_BWD: da = acc0, da' = acc1, the stored derivatives read from Z, Zd ->
+//               dz = Z da, dz' = Zd da + Z da'  -> A, Ad.
 struct EpiOut {
   float c0, c1;     // float32 outputs for C0 / C1
   float o0, o1;     // values for A / Ad
 };
 
+__device__ __forceinline__ EpiOut epi_bwd(float acc0, float acc1, float d1, float e, bool dual) {
+  EpiOut r;
+  r.c0 = acc0; r.c1 = acc1;
+  r.o0 = d1 * acc0;
+  r.o1 = dual ? e * acc0 + d1 * acc1 : 0.f;
+  return r;
+}
+
+// f, d1, d2 = phi, phi', phi'' at z
+__device__ __forceinline__ EpiOut epi_fwd(float f, float d1, float d2, float zd, bool dual) {
+  EpiOut r;
+  r.c0 = d1;
+  r.c1 = dual ? d2 * zd : d2;
+  r.o0 = f;
+  r.o1 = dual ? d1 * zd : 0.f;
+  return r;
+}
+
 __device__ __forceinline__ EpiOut epi_eval(const EpiParams& e, int m, int n, float acc0,
                                            float acc1, const float* bias0, const float* bias1,
                                            bool dual) {
-  EpiOut r;
   if (e.mode == EPI_ACT_BWD) {
-    const float z = e.Z[static_cast<int64_t>(m) * e.ldz + n];
-    float f, d1, d2;
-    act_eval(e.act, z, f, d1, d2);
-    r.c0 = acc0; r.c1 = acc1;
-    r.o0 = d1 * acc0;
-    r.o1 = dual ? d2 * e.Zd[static_cast<int64_t>(m) * e.ldz + n] * acc0 + d1 * acc1 : 0.f;
-    return r;
+    const int64_t at = static_cast<int64_t>(m) * e.ldz + n;
+    return epi_bwd(acc0, acc1, e.Z[at], dual ? e.Zd[at] : 0.f, dual);
   }
   const float z = acc0 + (bias0 ? bias0[n] : 0.f);
   const float zd = acc1 + (bias1 ? bias1[n] : 0.f);
-  r.c0 = z; r.c1 = zd;
   if (e.mode == EPI_ACT_FWD) {
     float f, d1, d2;
     act_eval(e.act, z, f, d1, d2);
-    r.o0 = f;
-    r.o1 = dual ? d1 * zd : 0.f;
-  } else {
-    r.o0 = r.o1 = 0.f;
+    return epi_fwd(f, d1, d2, zd, dual);
   }
+  EpiOut r;
+  r.c0 = z; r.c1 = zd;
+  r.o0 = r.o1 = 0.f;
   return r;
 }
 
@@ -102,31 +116,22 @@ __device__ __forceinline__ void act_eval_t(float z, float& f, float& d1, float& 
   }
 }
 
-// The per-element arithmetic of epi_eval_t on values already loaded: z, zd the stored
-// pre-activation and its tangent (EPI_ACT_BWD), b0, b1 the biases (0 when absent).
+// The per-element arithmetic of epi_eval_t on values already loaded: x0, x1 the stored
+// derivatives (EPI_ACT_BWD); b0, b1 the biases (0 when absent).
 template <int MODE, int ACT>
-__device__ __forceinline__ EpiOut epi_core_t(float acc0, float acc1, float z_in, float zd_in,
+__device__ __forceinline__ EpiOut epi_core_t(float acc0, float acc1, float x0, float x1,
                                              float b0, float b1, bool dual) {
-  EpiOut r;
-  if constexpr (MODE == EPI_ACT_BWD) {
+  if constexpr (MODE == EPI_ACT_BWD) return epi_bwd(acc0, acc1, x0, x1, dual);
+  const float z = acc0 + b0;
+  const float zd = acc1 + b1;
+  if constexpr (MODE == EPI_ACT_FWD) {
     float f, d1, d2;
-    act_eval_t<ACT>(z_in, f, d1, d2);
-    r.c0 = acc0; r.c1 = acc1;
-    r.o0 = d1 * acc0;
-    r.o1 = dual ? d2 * zd_in * acc0 + d1 * acc1 : 0.f;
-  } else {
-    const float z = acc0 + b0;
-    const float zd = acc1 + b1;
-    r.c0 = z; r.c1 = zd;
-    if constexpr (MODE == EPI_ACT_FWD) {
-      float f, d1, d2;
-      act_eval_t<ACT>(z, f, d1, d2);
-      r.o0 = f;
-      r.o1 = dual ? d1 * zd : 0.f;
-    } else {
-      r.o0 = r.o1 = 0.f;
-    }
+    act_eval_t<ACT>(z, f, d1, d2);
+    return epi_fwd(f, d1, d2, zd, dual);
   }
+  EpiOut r;
+  r.c0 = z; r.c1 = zd;
+  r.o0 = r.o1 = 0.f;
   return r;
 }
 

@@ -52,7 +52,7 @@ template <> __device__ __forceinline__ float to_f<__nv_bfloat16>(__nv_bfloat16 x
 }
 
 // LOSS: 0 squared, 1 softmax CE.  DUAL: tangent pass along u.
-template <typename T, int ACT, bool DUAL, int LOSS>
+template <typename T, bool DUAL, int LOSS>
 __global__ void __launch_bounds__(HEAD_THREADS) head_fused_kernel(const HeadArgs a) {
   pdl_entry();
   __shared__ float red[HEAD_WARPS][2 * kHeadMaxOut];
@@ -171,7 +171,6 @@ __global__ void __launch_bounds__(HEAD_THREADS) head_fused_kernel(const HeadArgs
   // ---- 3. head data product and the activation backward of the layer below ------------
   EpiParams e;
   e.mode = EPI_ACT_BWD;
-  e.act = ACT;
   e.Z = a.Z; e.Zd = a.Zd; e.ldz = a.ldz;
   T* dzp = static_cast<T*>(a.dz_prev) + static_cast<int64_t>(row) * a.ld_prev;
   T* dzdp = DUAL ? static_cast<T*>(a.dzd_prev) + static_cast<int64_t>(row) * a.ld_prev : nullptr;
@@ -187,22 +186,10 @@ __global__ void __launch_bounds__(HEAD_THREADS) head_fused_kernel(const HeadArgs
         if (DUAL) dad = fmaf(seed[1][j], wj, fmaf(seed[0][j], to_f<T>(u[j]), dad));
       }
     }
-    const EpiOut o = epi_eval_t<EPI_ACT_BWD, ACT>(e, row, k, da, dad, nullptr, nullptr, DUAL);
+    const EpiOut o = epi_eval_t<EPI_ACT_BWD, ACT_IDENT>(e, row, k, da, dad, nullptr, nullptr, DUAL);
     dzp[k] = to_t<T>(o.o0);
     if (DUAL) dzdp[k] = to_t<T>(o.o1);
   }
-}
-
-template <typename T, int ACT>
-cudaError_t launch_act(const HeadArgs& a, cudaStream_t s) {
-  const dim3 grid(a.rows), block(HEAD_THREADS);
-  const int lk = a.loss.loss;
-  if (a.dual) {
-    if (lk == 0) return launch_k(head_fused_kernel<T, ACT, true, 0>, grid, block, 0, s, a);
-    return launch_k(head_fused_kernel<T, ACT, true, 1>, grid, block, 0, s, a);
-  }
-  if (lk == 0) return launch_k(head_fused_kernel<T, ACT, false, 0>, grid, block, 0, s, a);
-  return launch_k(head_fused_kernel<T, ACT, false, 1>, grid, block, 0, s, a);
 }
 
 }  // namespace
@@ -215,13 +202,14 @@ cudaError_t head_fused(const HeadArgs& a, cudaStream_t s) {
   if (a.C < 1 || a.C > kHeadMaxOut || a.D < 1 || (a.loss.loss != 0 && a.loss.loss != 1) ||
       (a.loss.loss == 0 && !a.loss.Yf) || (a.loss.loss == 1 && !a.loss.Yi))
     return cudaErrorInvalidValue;
-  switch (a.act) {
-    case ACT_IDENT: return launch_act<T, ACT_IDENT>(a, s);
-    case ACT_TANH: return launch_act<T, ACT_TANH>(a, s);
-    case ACT_GELU: return launch_act<T, ACT_GELU>(a, s);
-    case ACT_SILU: return launch_act<T, ACT_SILU>(a, s);
+  const dim3 grid(a.rows), block(HEAD_THREADS);
+  const int lk = a.loss.loss;
+  if (a.dual) {
+    if (lk == 0) return launch_k(head_fused_kernel<T, true, 0>, grid, block, 0, s, a);
+    return launch_k(head_fused_kernel<T, true, 1>, grid, block, 0, s, a);
   }
-  return cudaErrorInvalidValue;
+  if (lk == 0) return launch_k(head_fused_kernel<T, false, 0>, grid, block, 0, s, a);
+  return launch_k(head_fused_kernel<T, false, 1>, grid, block, 0, s, a);
 }
 
 template cudaError_t head_fused<float>(const HeadArgs&, cudaStream_t);

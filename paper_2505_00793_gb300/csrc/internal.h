@@ -65,7 +65,8 @@ struct EpiParams {
   int mode = EPI_STORE;
   int act = ACT_IDENT;
   void* A = nullptr; void* Ad = nullptr; int lda = 0;
-  const float* Z = nullptr; const float* Zd = nullptr; int ldz = 0;   // EPI_ACT_BWD inputs
+  // EPI_ACT_BWD inputs: what EPI_ACT_FWD left in C0 and C1, phi'(z) and phi''(z) z'
+  const float* Z = nullptr; const float* Zd = nullptr; int ldz = 0;
 };
 
 // C[m][n] (+)= sum over selected terms of X[m][k] * Y[n][k]   (both operands K-major).
@@ -89,6 +90,12 @@ struct GemmArgs {
   bool a_mn = false, b_mn = false;
   int* status = nullptr;   // device status word (timeouts), may be null
 };
+
+// Whether the epilogue writes C1: a second accumulator, or the second derivative that a
+// primal forward epilogue leaves there.
+inline bool writes_c1(const GemmArgs& a) {
+  return (a.terms & (T_C1_A1B0 | T_C1_A0B1)) || a.epi.mode == EPI_ACT_FWD;
+}
 
 // tcgen05 bf16 GEMM (tc_gemm.cu).  Returns cudaSuccess or the launch error; sets *why on a
 // host-side rejection (bad alignment/ld) and returns cudaErrorInvalidValue.
@@ -160,12 +167,12 @@ constexpr int kHeadMaxOut = 16;
 struct HeadArgs {
   int rows = 0, D = 0, C = 0;      // example rows, head input width, head outputs
   bool dual = false;               // tangent pass along u
-  int act = ACT_IDENT;             // activation of the layer below the head
   const void* A = nullptr; const void* Ad = nullptr; int lda = 0;   // head inputs [rows][lda] (T)
   const void* W = nullptr; const void* U = nullptr; int ldw = 0;    // [D][ldw] operand copies (T)
   const float* bias = nullptr; const float* ubias = nullptr;        // nullable
   LossArgs loss;                   // targets, weights, outputs and the head seeds (dF, dFd, ldo)
-  const float* Z = nullptr; const float* Zd = nullptr; int ldz = 0;      // layer below: z, z'
+  const float* Z = nullptr; const float* Zd = nullptr; int ldz = 0;      // layer below: its stored
+                                                                         // derivatives
   void* dz_prev = nullptr; void* dzd_prev = nullptr; int ld_prev = 0;    // its seeds (T); null:
                                                                          // no data product
 };
@@ -241,14 +248,15 @@ void layer_update(const LayerTable& tab, const LayerUpdArgs& a, cudaStream_t s);
 
 void fill(float* p, int64_t n, float v, cudaStream_t s);
 
-// Reverse-over-reverse element kernels (MLP): dabar = dzbar phi'(z), zpart = dzbar phi''(z) da;
-// zbar = zpart + abar phi'(z).  T outputs row-major [rows][ld].
+// Reverse-over-reverse element kernels (MLP), from the derivatives D1 = phi'(z), D2 = phi''(z)
+// that the primal forward stored: dabar = dzbar D1, zpart = dzbar D2 da; zbar = zpart + abar D1.
+// T outputs row-major [rows][ld].
 template <typename T>
-void ror_fwd_elem(int act, const float* dzbar, const float* Z, const float* dA, int rows, int cols,
-                  T* dab, int ld, float* zpart, cudaStream_t s);
+void ror_fwd_elem(const float* dzbar, const float* D1, const float* D2, const float* dA, int rows,
+                  int cols, T* dab, int ld, float* zpart, cudaStream_t s);
 template <typename T>
-void ror_bwd_elem(int act, const float* zpart, const float* abar, const float* Z, int rows,
-                  int cols, T* zb, int ld, cudaStream_t s);
+void ror_bwd_elem(const float* zpart, const float* abar, const float* D1, int rows, int cols,
+                  T* zb, int ld, cudaStream_t s);
 
 // ---- fused dual attention (flash_attn.cu) -------------------------------------------------
 // Heads [BH][S][64] bf16 (q pre-scaled by 1/sqrt(64)), causal.  Forward: O (and O') float32

@@ -507,11 +507,12 @@ __global__ void __launch_bounds__(UPD_THREADS) layer_update_kernel(const LayerTa
   }
 }
 
-// Reverse-over-reverse, forward layer order: from dzbar (the adjoint of the backward's dz):
-//   dabar = dzbar phi'(z)  (T, row-major [rows][ld]),  zpart = dzbar phi''(z) da.
+// Reverse-over-reverse, forward layer order: from dzbar (the adjoint of the backward's dz)
+// and the stored derivatives D1 = phi'(z), D2 = phi''(z):
+//   dabar = dzbar D1  (T, row-major [rows][ld]),  zpart = dzbar D2 da.
 template <typename T>
-__global__ void ror_fwd_elem_kernel(int act, const float* __restrict__ dzbar,
-                                    const float* __restrict__ Z, const float* __restrict__ dA,
+__global__ void ror_fwd_elem_kernel(const float* __restrict__ dzbar, const float* __restrict__ D1,
+                                    const float* __restrict__ D2, const float* __restrict__ dA,
                                     int rows, int cols, T* __restrict__ dab, int ld,
                                     float* __restrict__ zpart) {
   pdl_entry();
@@ -520,18 +521,16 @@ __global__ void ror_fwd_elem_kernel(int act, const float* __restrict__ dzbar,
     const int r = blockIdx.y * TILE + i;
     if (r < rows && c < cols) {
       const int64_t o = static_cast<int64_t>(r) * cols + c;
-      float f, d1, d2;
-      act_eval(act, Z[o], f, d1, d2);
-      zpart[o] = dzbar[o] * d2 * dA[o];
-      dab[static_cast<int64_t>(r) * ld + c] = to_t<T>(dzbar[o] * d1);
+      zpart[o] = dzbar[o] * D2[o] * dA[o];
+      dab[static_cast<int64_t>(r) * ld + c] = to_t<T>(dzbar[o] * D1[o]);
     }
   }
 }
 
-// Reverse-over-reverse, reverse layer order:  zbar = zpart + abar phi'(z)  (T, [rows][ld]).
+// Reverse-over-reverse, reverse layer order:  zbar = zpart + abar D1  (T, [rows][ld]).
 template <typename T>
-__global__ void ror_bwd_elem_kernel(int act, const float* __restrict__ zpart,
-                                    const float* __restrict__ abar, const float* __restrict__ Z,
+__global__ void ror_bwd_elem_kernel(const float* __restrict__ zpart,
+                                    const float* __restrict__ abar, const float* __restrict__ D1,
                                     int rows, int cols, T* __restrict__ zb, int ld) {
   pdl_entry();
   const int c = blockIdx.x * TILE + threadIdx.x;
@@ -539,9 +538,7 @@ __global__ void ror_bwd_elem_kernel(int act, const float* __restrict__ zpart,
     const int r = blockIdx.y * TILE + i;
     if (r < rows && c < cols) {
       const int64_t o = static_cast<int64_t>(r) * cols + c;
-      float f, d1, d2;
-      act_eval(act, Z[o], f, d1, d2);
-      zb[static_cast<int64_t>(r) * ld + c] = to_t<T>(zpart[o] + abar[o] * d1);
+      zb[static_cast<int64_t>(r) * ld + c] = to_t<T>(zpart[o] + abar[o] * D1[o]);
     }
   }
 }
@@ -604,20 +601,20 @@ void layer_update(const LayerTable& tab, const LayerUpdArgs& args, cudaStream_t 
 }
 
 template <typename T>
-void ror_fwd_elem(int act, const float* dzbar, const float* Z, const float* dA, int rows, int cols,
-                  T* dab, int ld, float* zpart, cudaStream_t s) {
+void ror_fwd_elem(const float* dzbar, const float* D1, const float* D2, const float* dA, int rows,
+                  int cols, T* dab, int ld, float* zpart, cudaStream_t s) {
   if (rows <= 0 || cols <= 0) return;
   dim3 grid((cols + TILE - 1) / TILE, (rows + TILE - 1) / TILE);
-  launch_k(ror_fwd_elem_kernel<T>, dim3(grid), dim3(TILE, TROWS), 0, s, act, dzbar, Z, dA, rows,
+  launch_k(ror_fwd_elem_kernel<T>, dim3(grid), dim3(TILE, TROWS), 0, s, dzbar, D1, D2, dA, rows,
            cols, dab, ld, zpart);
 }
 
 template <typename T>
-void ror_bwd_elem(int act, const float* zpart, const float* abar, const float* Z, int rows,
-                  int cols, T* zb, int ld, cudaStream_t s) {
+void ror_bwd_elem(const float* zpart, const float* abar, const float* D1, int rows, int cols,
+                  T* zb, int ld, cudaStream_t s) {
   if (rows <= 0 || cols <= 0) return;
   dim3 grid((cols + TILE - 1) / TILE, (rows + TILE - 1) / TILE);
-  launch_k(ror_bwd_elem_kernel<T>, dim3(grid), dim3(TILE, TROWS), 0, s, act, zpart, abar, Z, rows,
+  launch_k(ror_bwd_elem_kernel<T>, dim3(grid), dim3(TILE, TROWS), 0, s, zpart, abar, D1, rows,
            cols, zb, ld);
 }
 
@@ -632,9 +629,9 @@ void fill(float* p, int64_t n, float v, cudaStream_t s) {
   template void fill_cols<T>(const ColFill&, int, cudaStream_t);                  \
   template void loss_seed<T>(const LossArgs&, cudaStream_t);                      \
   template void layer_update<T>(const LayerTable&, const LayerUpdArgs&, cudaStream_t);        \
-  template void ror_fwd_elem<T>(int, const float*, const float*, const float*, int, int, T*, int, \
-                                float*, cudaStream_t);                                            \
-  template void ror_bwd_elem<T>(int, const float*, const float*, const float*, int, int, T*, int,  \
+  template void ror_fwd_elem<T>(const float*, const float*, const float*, const float*, int, int, \
+                                T*, int, float*, cudaStream_t);                                  \
+  template void ror_bwd_elem<T>(const float*, const float*, const float*, int, int, T*, int,     \
                                 cudaStream_t);
 MF_INST(float)
 MF_INST(__nv_bfloat16)

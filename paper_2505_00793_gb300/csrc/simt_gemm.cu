@@ -17,7 +17,7 @@
 //    of up to 8 CTAs whose partial tiles meet in distributed shared memory; the sums run in
 //    a fixed order, so results are deterministic.
 // Measured against one 64 x 64 tile per block that ran a mask's terms one after the other
-// from single-buffered tiles: the five layers of a 784-1023-1023-500-10 Hessian-vector
+// from single-buffered tiles: the layers of a 784-1023-1023-500-10 Hessian-vector
 // product at 500 rows 8.31 -> 0.59 ms, four training steps of a 4 x 256 transformer
 // (1024 tokens) 65.8 -> 4.8 ms; large products run at 38-52 TFLOP/s (4096x4096x1024: the
 // FMA pipes active 71% of the time) where they ran at 2.
@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(32 * WM * WN * KS)
       }
     };
     if (p.C[0]) put(p.C[0] + bz * p.bsC[0], static_cast<int64_t>(gm) * p.ldc[0] + gn, c0, p.c_vec);
-    if (p.C[1] && dual) put(p.C[1] + bz * p.bsC[1], static_cast<int64_t>(gm) * p.ldc[1] + gn, c1, p.c_vec);
+    if (p.C[1]) put(p.C[1] + bz * p.bsC[1], static_cast<int64_t>(gm) * p.ldc[1] + gn, c1, p.c_vec);
     if (e.mode != EPI_STORE) {
       if (EA) put(EA, static_cast<int64_t>(gm) * e.lda + gn, o0, p.e_vec);
       if (dual && EAd) put(EAd, static_cast<int64_t>(gm) * e.lda + gn, o1, p.e_vec);
@@ -373,7 +373,7 @@ cudaError_t simt_gemm(const GemmArgs& a, cudaStream_t s) {
   p.B[0] = static_cast<const float*>(a.B0); p.ldb[0] = a.ldb0;
   p.B[1] = static_cast<const float*>(a.B1); p.ldb[1] = a.ldb1;
   p.C[0] = a.C0; p.ldc[0] = a.ldc0; p.bias[0] = a.bias0;
-  p.C[1] = a.C1; p.ldc[1] = a.ldc1; p.bias[1] = a.bias1;
+  p.C[1] = writes_c1(a) ? a.C1 : nullptr; p.ldc[1] = a.ldc1; p.bias[1] = a.bias1;
   p.epi = a.epi;
   p.a_mn = a.a_mn ? 1 : 0;
   p.b_mn = a.b_mn ? 1 : 0;

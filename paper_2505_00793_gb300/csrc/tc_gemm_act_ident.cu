@@ -1,6 +1,7 @@
 // Activation-epilogue instances of the tcgen05 dual GEMM for ACT_IDENT (forward: bias + phi,
-// phi' z'; backward: phi' da, phi'' z' da + phi' da'), one translation unit per activation so
-// that the instances compile in parallel.
+// phi' z' and the derivatives the backward needs), and the backward instance of every
+// activation (dz = phi' da, dz' = phi'' z' da + phi' da' from the derivatives the forward stored).
+// One translation unit per activation so that the instances compile in parallel.
 #include "tc_gemm_impl.cuh"
 
 namespace mf {

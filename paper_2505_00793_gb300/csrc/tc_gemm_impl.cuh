@@ -317,7 +317,7 @@ __device__ __forceinline__ void epilogue16(const TcParams& p, int row, int col0,
         for (int j = 0; j < 16; ++j) if (col0 + j < p.N) dst[j] = c0[j];
       }
     }
-    if (p.C1 && dual) {
+    if (p.C1) {
       float* dst = p.C1 + static_cast<int64_t>(row) * p.ldc1 + col0;
       if (full && !(p.ldc1 & 3) && !(reinterpret_cast<uintptr_t>(p.C1) & 15)) {
 #pragma unroll
@@ -414,7 +414,7 @@ __device__ __forceinline__ bool rows16_ok(const TcParams& p, int mode, bool dual
   auto al = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
   bool ok = true;
   if (p.C0) ok = ok && al(p.C0) && !(p.ldc0 & 3);
-  if (p.C1 && dual) ok = ok && al(p.C1) && !(p.ldc1 & 3);
+  if (p.C1) ok = ok && al(p.C1) && !(p.ldc1 & 3);
   if (mode != EPI_STORE) {
     if (p.epi.A) ok = ok && al(p.epi.A) && !(p.epi.lda & 7);
     if (p.epi.Ad && dual) ok = ok && al(p.epi.Ad) && !(p.epi.lda & 7);
@@ -446,15 +446,17 @@ __device__ __forceinline__ void rows_to_quads(uint8_t* stg, int lane, const floa
 
 // epilogue16 for a full chunk (col0 + 16 <= N) of the warp's 32 rows row0 .. row0 + 31.  Only
 // the accumulators change layout: they cross the per-warp buffer stg (STG_ROWS_BYTES) into
-// quads, in which the stored pre-activations of backward epilogues arrive (zq, zdq: loads
+// quads, in which the stored derivatives of backward epilogues arrive (zq, zdq: loads
 // already issued, see zrows_issue) and every output leaves, 8 rows x 64 bytes (float32) or
 // x 32 bytes (bf16) per warp store.  The biases load ahead of the arithmetic, without a
 // branch per element between the lane's sixteen independent chains.  The arithmetic per
 // element is epi_core_t's, as in epilogue16.  Rows at or past M are computed but not stored.
 // Moving every input and output through the buffer instead, with a bias test per element,
 // this epilogue was the longer role of short-K products: 8192 x 4096 x 1024 forward with GELU
-// about 115 -> 72 us (SiLU 130 -> 84, tanh 91 -> 62), dual GELU 178 -> 149 us, dual GELU
-// backward 191 -> 168 us.
+// about 115 -> 72 us (SiLU 130 -> 84, tanh 91 -> 62), dual GELU 178 -> 149 us.  The backward
+// multiplies by derivatives that the forward stored instead of evaluating the activation
+// again: its GEMM of the same shape 98 -> 44 us, dual 160 -> 119 us (erff and expf took 60
+// clocks per element of its eight warps).
 template <int MODE, int ACT, bool DUALE>
 __device__ __forceinline__ void epilogue16_rows_t(const TcParams& p, uint8_t* stg, int lane,
                                                   int row0, int col0, float (&v0)[16],
@@ -479,7 +481,7 @@ __device__ __forceinline__ void epilogue16_rows_t(const TcParams& p, uint8_t* st
   if constexpr (dual) rows_to_quads(stg, lane, v1, x1);
   auto rowp = [&](auto* base, int64_t ld) { return base ? base + row * ld + col : base; };
   float* const C0 = rowp(p.C0, p.ldc0);
-  float* const C1 = dual ? rowp(p.C1, p.ldc1) : nullptr;
+  float* const C1 = dual || MODE == EPI_ACT_FWD ? rowp(p.C1, p.ldc1) : nullptr;
   __nv_bfloat16 *A = nullptr, *Ad = nullptr;
   if constexpr (MODE != EPI_STORE) {
     A = rowp(static_cast<__nv_bfloat16*>(p.epi.A), p.epi.lda);
@@ -498,7 +500,7 @@ __device__ __forceinline__ void epilogue16_rows_t(const TcParams& p, uint8_t* st
     if (C0 && in)
       *reinterpret_cast<float4*>(C0 + 8 * i * static_cast<int64_t>(p.ldc0)) =
           make_float4(o[0].c0, o[1].c0, o[2].c0, o[3].c0);
-    if (dual && C1 && in)
+    if ((dual || MODE == EPI_ACT_FWD) && C1 && in)
       *reinterpret_cast<float4*>(C1 + 8 * i * static_cast<int64_t>(p.ldc1)) =
           make_float4(o[0].c1, o[1].c1, o[2].c1, o[3].c1);
     if constexpr (MODE != EPI_STORE) {
@@ -547,7 +549,7 @@ __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wa
 constexpr int STG_F32_BOX = 32 * 32 * 4;          // 4 KB
 constexpr int STG_BF16_BOX = 32 * 64 * 2;         // 4 KB
 // ... followed by the row-block buffer (STG_ROWS_BYTES) through which the backward
-// epilogues read the stored pre-activations.
+// epilogues read the stored derivatives.
 constexpr int STG_ZROWS = 4 * STG_F32_BOX + 2 * STG_BF16_BOX;
 constexpr int STG_WARP = STG_ZROWS + STG_ROWS_BYTES;              // 26 KB
 
@@ -567,7 +569,7 @@ __device__ __forceinline__ void epilogue_tma(const TcParams& p, const CUtensorMa
   uint8_t* sAd = sA + STG_BF16_BOX;
   uint8_t* sZ = stg + STG_ZROWS;
   const int sw = lane & 7;
-  // backward epilogues: the stored pre-activations of full chunks through sZ
+  // backward epilogues: the stored derivatives of full chunks through sZ
   bool zrows_ok = false;
   if constexpr (MODE == EPI_ACT_BWD) {
     auto al = [](const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15) == 0; };
@@ -975,7 +977,7 @@ struct EpiTile {
   }
 };
 
-// Stored inputs of the epilogue of four consecutive elements (m, n..n+3): the pre-activation
+// Stored inputs of the epilogue of four consecutive elements (m, n..n+3): the derivative
 // and its tangent (EPI_ACT_BWD) or the biases.
 struct EpiIn {
   float x0[4], x1[4];
@@ -1041,7 +1043,7 @@ __device__ __forceinline__ void epi_quad(const TcParams& p, int m, int n, const 
     }
   };
   if (p.C0) put(p.C0, p.ldc0, c0);
-  if (p.C1 && dual) put(p.C1, p.ldc1, c1);
+  if (p.C1) put(p.C1, p.ldc1, c1);
   if constexpr (MODE != EPI_STORE) {
     // row-major operand copies (16-byte aligned, ld a multiple of 8, n a multiple of 4)
     auto puth = [&](void* A, const float (&o)[4]) {
@@ -1371,7 +1373,7 @@ cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s, const char** why) {
   if (stages < 2) { *why = "tile does not fit shared memory"; return cudaErrorInvalidValue; }
   p.stages = stages;
   p.C0 = a.C0; p.ldc0 = a.ldc0; p.bias0 = a.bias0;
-  p.C1 = dual ? a.C1 : nullptr; p.ldc1 = a.ldc1; p.bias1 = a.bias1;
+  p.C1 = writes_c1(a) ? a.C1 : nullptr; p.ldc1 = a.ldc1; p.bias1 = a.bias1;
   p.epi = a.epi;
   p.status = a.status;
   p.wait_ns = g_wait_ns;
@@ -1615,7 +1617,7 @@ cudaError_t launch_cfg2(const GemmArgs& a, cudaStream_t s, const char** why) {
   p.stages = stages;
   p.split = 1;
   p.C0 = a.C0; p.ldc0 = a.ldc0; p.bias0 = a.bias0;
-  p.C1 = dual ? a.C1 : nullptr; p.ldc1 = a.ldc1; p.bias1 = a.bias1;
+  p.C1 = writes_c1(a) ? a.C1 : nullptr; p.ldc1 = a.ldc1; p.bias1 = a.bias1;
   p.epi = a.epi;
   p.status = a.status;
   p.wait_ns = g_wait_ns;

@@ -33,8 +33,7 @@ int g_gemm_persist = 2;
 namespace {
 
 // Epilogue warps per CTA: twelve (three per TMEM lane quadrant) where the epilogue is the
-// longer role, eight for the backward epilogues, whose prefetched pre-activations need the
-// registers of a 320-thread CTA.
+// longer role, eight for the backward epilogues, which only load and multiply.
 template <int MODE>
 __host__ __device__ constexpr int epi_warps_p() { return MODE == EPI_ACT_BWD ? 8 : 12; }
 template <int MODE>
@@ -386,22 +385,15 @@ __global__ void __launch_bounds__(threads_p<MODE>(), 1)
       p.C0 = C0base ? C0base + bz * p.bsC0 : nullptr;
       p.C1 = C1base ? C1base + bz * p.bsC1 : nullptr;
       const uint32_t taddr = tbase + lane_off + static_cast<uint32_t>(set * pp.set_cols);
-      // backward epilogues: the next full chunk's stored pre-activations load while this
-      // chunk is computed
-      ZRows zq, zdq, zq_n, zdq_n;
-      auto zissue = [&](int c, ZRows& a, ZRows& b) {
-        if (rows_ok && n0 + c + 16 <= p.N) {
-          zrows_issue(a, lane, m0 + q * 32, p.M, p.epi.Z, p.epi.ldz, n0 + c);
-          if (dual) zrows_issue(b, lane, m0 + q * 32, p.M, p.epi.Zd, p.epi.ldz, n0 + c);
-        }
-      };
-      if constexpr (MODE == EPI_ACT_BWD) zissue(c_begin, zq_n, zdq_n);
 #pragma unroll 1
       for (int c = c_begin; c < c_end; c += CSTEP) {
+        // backward epilogues: the chunk's stored derivatives load with the accumulators
+        ZRows zq, zdq;
         if constexpr (MODE == EPI_ACT_BWD) {
-          zq = zq_n;
-          zdq = zdq_n;
-          if (c + CSTEP < c_end) zissue(c + CSTEP, zq_n, zdq_n);
+          if (rows_ok && n0 + c + 16 <= p.N) {
+            zrows_issue(zq, lane, m0 + q * 32, p.M, p.epi.Z, p.epi.ldz, n0 + c);
+            if (dual) zrows_issue(zdq, lane, m0 + q * 32, p.M, p.epi.Zd, p.epi.ldz, n0 + c);
+          }
         }
         float v0[16], v1[16];
         ld_acc16<BN>(taddr, 0, p.nsub, c, v0);
@@ -502,7 +494,7 @@ cudaError_t launch_cfg2p(const GemmArgs& a, cudaStream_t s, const char** why) {
   p.stages = stages;
   p.split = 1;
   p.C0 = a.C0; p.ldc0 = a.ldc0; p.bias0 = a.bias0;
-  p.C1 = dual ? a.C1 : nullptr; p.ldc1 = a.ldc1; p.bias1 = a.bias1;
+  p.C1 = writes_c1(a) ? a.C1 : nullptr; p.ldc1 = a.ldc1; p.bias1 = a.bias1;
   p.epi = a.epi;
   p.status = a.status;
   p.wait_ns = g_wait_ns;
@@ -592,13 +584,8 @@ cudaError_t tc_gemm_persist(const GemmArgs& a, cudaStream_t s, const char** why,
       case ACT_GELU: return launch_bn_p<EPI_ACT_FWD, ACT_GELU>(a, s, why, bn);
       case ACT_SILU: return launch_bn_p<EPI_ACT_FWD, ACT_SILU>(a, s, why, bn);
     }
-  } else if (a.epi.mode == EPI_ACT_BWD) {
-    switch (act) {
-      case ACT_IDENT: return launch_bn_p<EPI_ACT_BWD, ACT_IDENT>(a, s, why, bn);
-      case ACT_TANH: return launch_bn_p<EPI_ACT_BWD, ACT_TANH>(a, s, why, bn);
-      case ACT_GELU: return launch_bn_p<EPI_ACT_BWD, ACT_GELU>(a, s, why, bn);
-      case ACT_SILU: return launch_bn_p<EPI_ACT_BWD, ACT_SILU>(a, s, why, bn);
-    }
+  } else if (a.epi.mode == EPI_ACT_BWD) {   // from stored derivatives, whatever the activation
+    return launch_bn_p<EPI_ACT_BWD, ACT_IDENT>(a, s, why, bn);
   }
   *why = "unknown epilogue mode or activation";
   return cudaErrorInvalidValue;
