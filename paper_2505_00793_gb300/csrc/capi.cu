@@ -9,6 +9,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <type_traits>
@@ -413,6 +414,64 @@ struct Exec {
            h->dims[h->L] <= mf::kHeadMaxOut;
   }
 
+  // Small float32 models run as one block's program (small_program in kernels.cu): every
+  // operation below is recorded instead of launched, and the program runs, with the workspace
+  // in shared memory, when it is full or the call ends (flush).  Above the limits one block is
+  // slower than launches that spread over the GPU (launches -> program, us: 32-32-10 at B = 16
+  // meta-gradient 190 -> 142, HVP 29 -> 26; beyond them 100-35-10 at B = 8 HVP 32 -> 33,
+  // 60-50-10 at B = 16 31 -> 40, 40-48-10 at B = 32 31 -> 48).  The chain loss and the opt-in
+  // fused head are not recorded.
+  std::unique_ptr<mf::SmallProgram> prog;
+  static constexpr int64_t kSmallParams = 2048, kSmallWork = 20480;
+  bool small_model() const {
+    if (!std::is_same<T, float>::value || h->md.loss == MF_LOSS_CHAIN_MSE || p.head_bufs ||
+        h->P > kSmallParams || p.bytes > mf::kSmallImage)
+      return false;
+    int64_t work = 0;
+    for (int l = 0; l < h->L; ++l)
+      work = std::max(work, static_cast<int64_t>(p.rows) * (h->dims[l] + 1) * h->dims[l + 1]);
+    return work <= kSmallWork;
+  }
+  template <typename A>
+  bool record(mf::SmallKind kind, const A& a) {
+    if (!prog) return false;
+    if (prog->n == mf::kSmallOps) {
+      prog->save = 1;
+      flush();
+      prog->load = 1;
+      prog->save = 0;
+    }
+    prog->add(kind, a);
+    return true;
+  }
+  void flush() {
+    if (!prog || prog->n == 0) return;
+    const cudaError_t e = mf::small_program(*prog, s);
+    prog->n = 0;
+    launched();
+    chk(e, "small model program");
+  }
+  void chk(cudaError_t e, const char* what) {
+    if (e != cudaSuccess && st == MF_OK) {
+      st = MF_ERR_CUDA;
+      h->err = std::string(what) + ": " + cudaGetErrorString(e);
+    }
+  }
+  // dst[0..n) = src[0..n), or zeros
+  void copy(float* dst, const float* src, int64_t n) {
+    if (record(mf::SMALL_COPY, mf::SmallCopy{dst, src, 1, static_cast<int>(n), 0, 0, 0.f})) return;
+    chk(cudaMemcpyAsync(dst, src, n * 4, cudaMemcpyDeviceToDevice, s), "copy");
+  }
+  void zero(float* dst, int64_t n) {
+    if (record(mf::SMALL_COPY, mf::SmallCopy{dst, nullptr, 1, static_cast<int>(n), 0, 0, 0.f})) return;
+    chk(cudaMemsetAsync(dst, 0, n * 4, s), "clear");
+  }
+  void sum(const float* x, int n, float scale, float* out) {
+    if (record(mf::SMALL_SUM, mf::SmallSum{x, out, n, scale})) return;
+    mf::sum_scaled(x, n, scale, out, s);
+    launched();
+  }
+
   Exec(mf_ctx* h_, const Plan& p_, cudaStream_t s_)
       : h(h_), p(p_), s(s_), base(static_cast<char*>(h_->ws)) {
     tab.n = h->L;
@@ -430,6 +489,12 @@ struct Exec {
       tab.U[l] = at<T>(p.o_Ub[l]);
     }
     tab.tile0[h->L] = tiles;
+    if (small_model()) {
+      prog.reset(new mf::SmallProgram());
+      prog->tab = tab;
+      prog->ws = base;
+      prog->ws_bytes = static_cast<int>(p.bytes);
+    }
   }
 
   template <typename U> U* at(size_t off) const { return reinterpret_cast<U*>(base + off); }
@@ -450,7 +515,7 @@ struct Exec {
   void launched(int n = 1) { h->launches += n; }
 
   // Fork the side stream off the working stream / join it back (see mf_ctx::sstream).
-  bool can_fork() const { return h->concurrent && h->sstream && h->ev_fork && h->ev_join; }
+  bool can_fork() const { return !prog && h->concurrent && h->sstream && h->ev_fork && h->ev_join; }
   void fork() {
     if (cudaEventRecord(h->ev_fork, s) != cudaSuccess ||
         cudaStreamWaitEvent(h->sstream, h->ev_fork, 0) != cudaSuccess) {
@@ -468,6 +533,7 @@ struct Exec {
     if (st != MF_OK) return;
     const cudaStream_t s = on ? on : this->s;
     g.status = h->d_status;
+    if (record(mf::SMALL_GEMM, g)) return;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     unsigned ev_flags = cudaEventRecordDefault;
     const bool tc = h->bf16;
@@ -513,11 +579,23 @@ struct Exec {
         f.value[f.n] = 0.f; ++f.n;
       }
     }
+    if (prog) {
+      for (int i = 0; i < f.n; ++i)
+        record(mf::SMALL_COPY, mf::SmallCopy{static_cast<float*>(f.dst[i]) + f.col[i], nullptr, p.rows,
+                                             1, f.ld[i], 0, f.value[i]});
+      return;
+    }
     mf::fill_cols<T>(f, p.rows, s);
     launched();
   }
 
   void update(const mf::LayerUpdArgs& a) {
+    if (prog) {
+      mf::LayerUpdArgs b = a;
+      b.vec_ok = mf::update_vec_ok(a);
+      record(mf::SMALL_UPDATE, b);
+      return;
+    }
     mf::layer_update<T>(tab, a, s);
     launched();
   }
@@ -530,7 +608,7 @@ struct Exec {
   // layers' updates are independent of each other and of the layers still in the pass.
   const mf::LayerUpdArgs* upd_after = nullptr;
   bool layer_updates_ok() const {
-    return h->layer_updates && h->ustream && h->ev_u_in && h->ev_u_out;
+    return !prog && h->layer_updates && h->ustream && h->ev_u_in && h->ev_u_out;
   }
   void update_layer(const mf::LayerUpdArgs& a, int l) {
     mf::LayerTable t1;
@@ -581,11 +659,13 @@ struct Exec {
     const int din0 = h->dims[0];
     const size_t es = sizeof(T);
     // inputs into the augmented layer-0 activations (the bias column is already set)
-    if (cudaMemcpy2DAsync(at<T>(p.o_A[0]), p.lda[0] * es, xv, din0 * es, din0 * es, rows,
-                          cudaMemcpyDeviceToDevice, s) != cudaSuccess && st == MF_OK) {
-      st = MF_ERR_CUDA;
-      h->err = "input copy failed";
-    }
+    if (!prog)
+      chk(cudaMemcpy2DAsync(at<T>(p.o_A[0]), p.lda[0] * es, xv, din0 * es, din0 * es, rows,
+                            cudaMemcpyDeviceToDevice, s),
+          "input copy");
+    else
+      record(mf::SMALL_COPY, mf::SmallCopy{at<float>(p.o_A[0]), static_cast<const float*>(xv), rows,
+                                           din0, p.lda[0], din0, 0.f});
     for (int l = 0; l < h->L; ++l) {
       if (l == h->L - 1 && fused_head()) break;   // the output layer runs in loss()
       const int din = h->dims[l], dout = h->dims[l + 1];
@@ -646,6 +726,7 @@ struct Exec {
       head(rows, dual, a, fwd_theta, fwd_u);
       return;
     }
+    if (record(mf::SMALL_LOSS, a)) return;
     mf::loss_seed<T>(a, s);
     launched();
   }
@@ -800,10 +881,15 @@ struct Exec {
       g.bias0 = h->md.has_bias ? u + h->boff[l] : nullptr;
       gemm(g);
       if (l + 1 < L) {
-        mf::ror_fwd_elem<T>(at<float>(p.o_DZB), at<float>(p.o_Z[l]), at<float>(p.o_Zd[l]),
-                            at<float>(p.o_SA[l + 1]), rows, dout, at<T>(p.o_DAB[l]), p.lda[l + 1],
-                            at<float>(p.o_ZP[l]), s);
-        launched();
+        if (!record(mf::SMALL_ROR_FWD,
+                    mf::SmallRor{at<float>(p.o_DZB), at<float>(p.o_Z[l]), at<float>(p.o_Zd[l]),
+                                 at<float>(p.o_SA[l + 1]), at<float>(p.o_ZP[l]),
+                                 at<float>(p.o_DAB[l]), rows, dout, p.lda[l + 1]})) {
+          mf::ror_fwd_elem<T>(at<float>(p.o_DZB), at<float>(p.o_Z[l]), at<float>(p.o_Zd[l]),
+                              at<float>(p.o_SA[l + 1]), rows, dout, at<T>(p.o_DAB[l]), p.lda[l + 1],
+                              at<float>(p.o_ZP[l]), s);
+          launched();
+        }
       } else {
         // loss Hessian along dzbar (this is the forward tangent of the logits): zbar_{L-1},
         // the per-example directional losses and the weight meta-gradient
@@ -825,17 +911,23 @@ struct Exec {
           a.tape = at<float>(p.o_CH);
           a.ror = 2;
         }
-        mf::loss_seed<T>(a, s);
-        launched();
+        if (!record(mf::SMALL_LOSS, a)) {
+          mf::loss_seed<T>(a, s);
+          launched();
+        }
       }
     }
     // adjoint of the forward pass, layers L-1..0
     for (int l = L - 1; l >= 0; --l) {
       const int din = h->dims[l], dout = h->dims[l + 1];
       if (l + 1 < L) {
-        mf::ror_bwd_elem<T>(at<float>(p.o_ZP[l]), at<float>(p.o_AB), at<float>(p.o_Z[l]), rows,
-                            dout, at<T>(p.o_ZB), ld8(dout), s);
-        launched();
+        if (!record(mf::SMALL_ROR_BWD,
+                    mf::SmallRor{at<float>(p.o_AB), at<float>(p.o_Z[l]), nullptr, nullptr,
+                                 at<float>(p.o_ZP[l]), at<float>(p.o_ZB), rows, dout, ld8(dout)})) {
+          mf::ror_bwd_elem<T>(at<float>(p.o_ZP[l]), at<float>(p.o_AB), at<float>(p.o_Z[l]), rows,
+                              dout, at<T>(p.o_ZB), ld8(dout), s);
+          launched();
+        }
       }
       // (H v)_{W_l, b_l} = [a_{l-1}^T; 1] zbar_l + [dabar_{l-1}^T; 0] dz_l
       GemmArgs g;
@@ -1106,9 +1198,9 @@ mf_status meta_grad_run(X& ex, const mf_loop_desc* lp, const float* theta0, cons
   auto theta_at = [&](int t) { return ex.theta_slot(st.theta_idx(t)); };
   auto m_at = [&](int t) { return ex.m_slot(st.m_idx(t)); };   // m_t, t >= 1
   const bool scalar_lr = lp->meta_kind & MF_META_SCALAR_LOGLR;
-  MF_CUDA(h, cudaMemcpyAsync(theta_at(0), theta0, h->P * 4, cudaMemcpyDeviceToDevice, s));
+  ex.copy(theta_at(0), theta0, h->P);
   const int64_t ne = n_eta_of(h, lp);
-  if (ne > 0) MF_CUDA(h, cudaMemsetAsync(d_eta, 0, ne * 4, s));
+  if (ne > 0) ex.zero(d_eta, ne);
   ex.prepare();
 
   // 1. rollout into the checkpoint store; the last segment stays in the segment slots
@@ -1126,10 +1218,7 @@ mf_status meta_grad_run(X& ex, const mf_loop_desc* lp, const float* theta0, cons
   ex.forward(Bo, outer_x, thT, nullptr, false);
   ex.loss(Bo, false, outer_y, nullptr, nullptr, ex.l_buf(), nullptr, nullptr);
   ex.backward(Bo, false, nullptr, tbar);
-  if (outer_loss) {
-    mf::sum_scaled(ex.l_buf(), Bo, 1.f / Bo, outer_loss, s);
-    ex.launched();
-  }
+  if (outer_loss) ex.sum(ex.l_buf(), Bo, 1.f / Bo, outer_loss);
   float* d_plr = lr.off_plr >= 0 ? d_eta + lr.off_plr : nullptr;
   // Adam: reverse of inner step j from its stored outputs; u = g-bar_j, and the cotangents of
   // m_j, v_j replace those of m_{j+1}, v_{j+1} in place
@@ -1233,11 +1322,9 @@ mf_status meta_grad_run(X& ex, const mf_loop_desc* lp, const float* theta0, cons
     if (!per_layer) ex.update(a);
     if (ex.st != MF_OK) return ex.st;
   }
-  if (scalar_lr) {
-    mf::sum_scaled(part, T * nb, 1.f, d_eta + lr.off_slr, s);
-    ex.launched();
-  }
-  if (d_theta0) MF_CUDA(h, cudaMemcpyAsync(d_theta0, tbar, h->P * 4, cudaMemcpyDeviceToDevice, s));
+  if (scalar_lr) ex.sum(part, T * nb, 1.f, d_eta + lr.off_slr);
+  if (d_theta0) ex.copy(d_theta0, tbar, h->P);
+  ex.flush();
   MF_CUDA(h, cudaGetLastError());
   return ex.st;
 }
@@ -1293,9 +1380,9 @@ mf_status meta_grad_run_binomial(X& ex, const mf_loop_desc* lp, const float* the
   const BinSlots sl{&st};
   const mf::RevolveSchedule rs = mf::revolve_schedule(T, st.bin);
   const bool scalar_lr = lp->meta_kind & MF_META_SCALAR_LOGLR;
-  MF_CUDA(h, cudaMemcpyAsync(sl.theta(ex, 0), theta0, h->P * 4, cudaMemcpyDeviceToDevice, s));
+  ex.copy(sl.theta(ex, 0), theta0, h->P);
   const int64_t ne = n_eta_of(h, lp);
-  if (ne > 0) MF_CUDA(h, cudaMemsetAsync(d_eta, 0, ne * 4, s));
+  if (ne > 0) ex.zero(d_eta, ne);
   ex.prepare();
 
   // 1. rollout S_0 -> S_T, leaving S_t in slot keep[t] for the schedule's snapshots
@@ -1322,10 +1409,7 @@ mf_status meta_grad_run_binomial(X& ex, const mf_loop_desc* lp, const float* the
   ex.forward(Bo, outer_x, sl.theta(ex, sT), nullptr, false);
   ex.loss(Bo, false, outer_y, nullptr, nullptr, ex.l_buf(), nullptr, nullptr);
   ex.backward(Bo, false, nullptr, tbar);
-  if (outer_loss) {
-    mf::sum_scaled(ex.l_buf(), Bo, 1.f / Bo, outer_loss, s);
-    ex.launched();
-  }
+  if (outer_loss) ex.sum(ex.l_buf(), Bo, 1.f / Bo, outer_loss);
   float* d_plr = lr.off_plr >= 0 ? d_eta + lr.off_plr : nullptr;
   float* pend_m = st.adam ? ex.m_slot(st.bin_pend()) : nullptr;
   float* pend_v = st.adam ? ex.m_slot(st.bin_pend() + 1) : nullptr;
@@ -1352,8 +1436,8 @@ mf_status meta_grad_run_binomial(X& ex, const mf_loop_desc* lp, const float* the
   };
   bool adam_pending = false, pend_bar_in = false;
   auto defer_adam = [&](int slot, bool bar_in) {
-    MF_CUDA(h, cudaMemcpyAsync(pend_m, sl.m(ex, slot), h->P * 4, cudaMemcpyDeviceToDevice, s));
-    MF_CUDA(h, cudaMemcpyAsync(pend_v, sl.v(ex, slot), h->P * 4, cudaMemcpyDeviceToDevice, s));
+    ex.copy(pend_m, sl.m(ex, slot), h->P);
+    ex.copy(pend_v, sl.v(ex, slot), h->P);
     adam_pending = true;
     pend_bar_in = bar_in;
     return MF_OK;
@@ -1451,11 +1535,9 @@ mf_status meta_grad_run_binomial(X& ex, const mf_loop_desc* lp, const float* the
       if (e != MF_OK) return e;
     }
   }
-  if (scalar_lr) {
-    mf::sum_scaled(part, T * nb, 1.f, d_eta + lr.off_slr, s);
-    ex.launched();
-  }
-  if (d_theta0) MF_CUDA(h, cudaMemcpyAsync(d_theta0, tbar, h->P * 4, cudaMemcpyDeviceToDevice, s));
+  if (scalar_lr) ex.sum(part, T * nb, 1.f, d_eta + lr.off_slr);
+  if (d_theta0) ex.copy(d_theta0, tbar, h->P);
+  ex.flush();
   MF_CUDA(h, cudaGetLastError());
   return ex.st;
 }
@@ -1465,13 +1547,15 @@ mf_status rollout_run(X& ex, const mf_loop_desc* lp, const float* theta0, const 
                       const void* inner_x, const void* inner_y, float* thetaT) {
   mf_ctx* h = ex.h;
   const LrSel lr = lr_select(h, lp, eta);
-  MF_CUDA(h, cudaMemcpyAsync(ex.theta_slot(0), theta0, h->P * 4, cudaMemcpyDeviceToDevice, ex.s));
+  ex.copy(ex.theta_slot(0), theta0, h->P);
   ex.prepare();
   float* thT = nullptr;
   rollout_plain(ex, lp, eta, inner_x, inner_y, lr, &thT);
   if (ex.st != MF_OK) return ex.st;
-  MF_CUDA(h, cudaMemcpyAsync(thetaT, thT, h->P * 4, cudaMemcpyDeviceToDevice, ex.s));
-  return MF_OK;
+  ex.copy(thetaT, thT, h->P);
+  ex.flush();
+  MF_CUDA(h, cudaGetLastError());
+  return ex.st;
 }
 
 template <typename X>
@@ -1489,6 +1573,7 @@ mf_status hvp_run(X& ex, int B, const float* theta, const void* x, const void* y
     ex.loss(B, true, y, nullptr, ex_w, nullptr, tl, nullptr);
     ex.backward(B, true, Hv, grad);
   }
+  ex.flush();
   MF_CUDA(h, cudaGetLastError());
   return ex.st;
 }

@@ -220,6 +220,16 @@ struct DecExec {
     }
   }
 
+  void copy(float* dst, const float* src, int64_t n) {
+    chk_cuda(cudaMemcpyAsync(dst, src, n * 4, cudaMemcpyDeviceToDevice, s), "copy");
+  }
+  void zero(float* dst, int64_t n) { chk_cuda(cudaMemsetAsync(dst, 0, n * 4, s), "clear"); }
+  void sum(const float* x, int n, float scale, float* out) {
+    mf::sum_scaled(x, n, scale, out, s);
+    launched();
+  }
+  void flush() {}
+
   // index of a cast tensor in `tens`
   int tidx(int64_t off) const {
     for (int i = 0; i < static_cast<int>(tens.size()); ++i)

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
+#include <string.h>
 
 #include <mutex>
 
@@ -245,6 +246,50 @@ struct LayerUpdArgs {
 };
 template <typename T>
 void layer_update(const LayerTable& tab, const LayerUpdArgs& a, cudaStream_t s);
+
+bool update_vec_ok(const LayerUpdArgs& a);
+
+// A call of a small float32 MLP as one kernel (kernels.cu): the operations that the executor
+// would launch, recorded in order and run by one block.
+enum SmallKind : int {
+  SMALL_GEMM = 0, SMALL_LOSS, SMALL_UPDATE, SMALL_COPY, SMALL_SUM, SMALL_ROR_FWD, SMALL_ROR_BWD
+};
+struct SmallCopy {   // dst[r * ldd + c] = src[r * lds + c] (src null: value)
+  float* dst; const float* src;
+  int rows, cols, ldd, lds;
+  float value;
+};
+struct SmallSum { const float* x; float* out; int n; float scale; };
+struct SmallRor {    // x: dzbar (forward order) or abar; out: dabar or zbar, rows of ld floats
+  const float *x, *D1, *D2, *dA;
+  float *zpart, *out;
+  int rows, cols, ld;
+};
+struct alignas(8) SmallOp {
+  int kind;
+  alignas(8) unsigned char data[280];
+};
+static_assert(sizeof(GemmArgs) <= 280 && sizeof(LossArgs) <= 280 && sizeof(LayerUpdArgs) <= 280,
+              "an operation's arguments fit a program slot");
+// The program travels as a kernel parameter (32764 bytes at most).
+constexpr int kSmallOps = 96;
+constexpr int kSmallImage = 160 * 1024;   // largest workspace that is moved to shared memory
+struct alignas(16) SmallProgram {
+  LayerTable tab;
+  void* ws = nullptr;     // the workspace (ws_bytes, a multiple of 16)
+  int ws_bytes = 0;
+  int load = 0, save = 0; // the workspace enters from / leaves to global memory
+  int n = 0;
+  alignas(16) SmallOp op[kSmallOps];
+  template <typename A>
+  void add(SmallKind kind, const A& a) {
+    op[n].kind = kind;
+    memcpy(op[n].data, &a, sizeof(A));
+    ++n;
+  }
+};
+static_assert(sizeof(SmallProgram) <= 32764, "the program fits the kernel parameters");
+cudaError_t small_program(const SmallProgram& prog, cudaStream_t s);
 
 void fill(float* p, int64_t n, float v, cudaStream_t s);
 

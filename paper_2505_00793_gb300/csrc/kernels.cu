@@ -12,7 +12,9 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 #include <math.h>
+#include <stddef.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "device_math.cuh"
 #include "internal.h"
@@ -48,12 +50,7 @@ __device__ __forceinline__ float warp_max(float v) {
 // One warp per example row.  Squared loss l = 1/2 mean_o (f - y)^2; softmax CE
 // l = logsumexp(f) - f_y.  Seeds scaled by w_b / B.
 template <typename T>
-__global__ void loss_seed_kernel(const LossArgs a) {
-  pdl_entry();
-  const int warps = blockDim.x >> 5;
-  const int row = blockIdx.x * warps + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (row >= a.rows) return;
+__device__ __forceinline__ void loss_seed_row(const LossArgs& a, int row, int lane) {
   const int C = a.cols;
   const float* f = a.F + static_cast<int64_t>(row) * C;
   const float* fd = a.Fd ? a.Fd + static_cast<int64_t>(row) * C : nullptr;
@@ -109,6 +106,13 @@ __global__ void loss_seed_kernel(const LossArgs a) {
     if (a.ld) a.ld[row] = ld;
     if (a.d_eta && a.eta_w) a.d_eta[row] = sg * (1.f - sg) * ld * a.inv_norm;
   }
+}
+
+template <typename T>
+__global__ void loss_seed_kernel(const LossArgs a) {
+  pdl_entry();
+  const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (row < a.rows) loss_seed_row<T>(a, row, threadIdx.x & 31);
 }
 
 // Motivating example of Section 3 (Eq. 8): the model output is f = x theta followed by the
@@ -348,24 +352,24 @@ __device__ __forceinline__ void st_copy(T* W, int64_t e0, int dout, int din, int
   }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(UPD_THREADS) layer_update_kernel(const LayerTable tab,
-                                                                   const LayerUpdArgs a) {
-  pdl_entry();
-  __shared__ float red[UPD_THREADS / 32];
-  // the layer of this block: the last l with tile0[l] <= blockIdx.x (binary search)
+// Block blk of the update over the whole vector, by UPD_THREADS threads tid (red: one float a
+// warp; sync: their barrier).
+template <typename T, class Sync>
+__device__ __forceinline__ void layer_update_block(const LayerTable& tab, const LayerUpdArgs& a,
+                                                   int blk, int tid, float* red, Sync sync) {
+  // the layer of this block: the last l with tile0[l] <= blk (binary search)
   int l = 0;
   {
     int hi = tab.n - 1;
     while (l < hi) {
       const int mid = (l + hi + 1) >> 1;
-      if (static_cast<int>(blockIdx.x) >= tab.tile0[mid]) l = mid;
+      if (blk >= tab.tile0[mid]) l = mid;
       else hi = mid - 1;
     }
   }
   const int dout = tab.dout[l], din = tab.din[l];
   const int64_t n = static_cast<int64_t>(tab.rows[l]) * dout;
-  const int64_t e0 = (static_cast<int64_t>(blockIdx.x - tab.tile0[l]) * UPD_THREADS + threadIdx.x) * 4;
+  const int64_t e0 = (static_cast<int64_t>(blk - tab.tile0[l]) * UPD_THREADS + tid) * 4;
   const bool cast_w = (a.mode == LU_ROLLOUT) || (a.mode == LU_CAST && !a.cast_src_to_u) ||
                       (a.mode == LU_ADJOINT && a.cast_src);
   const bool cast_u = (a.mode == LU_CAST && a.cast_src_to_u) || (a.mode == LU_ADJOINT && a.u_out);
@@ -497,14 +501,24 @@ __global__ void __launch_bounds__(UPD_THREADS) layer_update_kernel(const LayerTa
   if (bad && a.status) atomicMax(a.status, DEV_NONFINITE);
   if (a.partials) {   // one deterministic partial sum per block (scalar log-lr)
     acc = warp_sum(acc);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      float v = threadIdx.x < UPD_THREADS / 32 ? red[threadIdx.x] : 0.f;
+    if ((tid & 31) == 0) red[tid >> 5] = acc;
+    sync();
+    if (tid < 32) {
+      float v = tid < UPD_THREADS / 32 ? red[tid] : 0.f;
       v = warp_sum(v);
-      if (threadIdx.x == 0) a.partials[blockIdx.x] = v;
+      if (tid == 0) a.partials[blk] = v;
     }
+    sync();   // red may be used again
   }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(UPD_THREADS) layer_update_kernel(const LayerTable tab,
+                                                                   const LayerUpdArgs a) {
+  pdl_entry();
+  __shared__ float red[UPD_THREADS / 32];
+  layer_update_block<T>(tab, a, static_cast<int>(blockIdx.x), static_cast<int>(threadIdx.x), red,
+                        [] { __syncthreads(); });
 }
 
 // Reverse-over-reverse, forward layer order: from dzbar (the adjoint of the backward's dz)
@@ -550,7 +564,201 @@ __global__ void fill_kernel(float* p, int64_t n, float v) {
     p[i] = v;
 }
 
+// ---- small float32 models: a whole call as one block's program ---------------------------
+// Every operation of a small MLP's call takes one block a fraction of a microsecond, and a
+// launch of its own three: the launches, not the work, are what such a call costs.  The block
+// walks the recorded operations in order with a barrier between them.  The call's workspace
+// lives in the block's shared memory (pointers into the workspace are moved there when the
+// program is read): from global memory, whose lines a store drops from L1, each operation
+// waited two round trips to L2.  Each is the operation of the kernel it stands for: the loss
+// and update share their device code, a GEMM is one output per thread with its products added
+// in K order.  What is left is the instructions of one block: splitting K over lanes or more
+// threads per block issued more of them and ran slower.
+// 16-32-1 at B = 8, T = 4 (70 operations): meta-gradient 185 us as launches, 108 us with the
+// workspace in global memory, 85 us; its Hessian-vector product 27 -> 17 us.
+constexpr int SP_THREADS = 512, SP_GROUPS = SP_THREADS / UPD_THREADS;
+static_assert(SP_THREADS >= kSmallOps && SP_THREADS >= kMaxLayers, "a thread per operation");
+
+__device__ __forceinline__ void small_gemm(const GemmArgs& g) {
+  const bool dual = (g.terms & (T_C1_A1B0 | T_C1_A0B1)) != 0;
+  const int K = g.K, N = g.N, total = g.M * N;
+  const int da = g.a_mn ? g.lda0 : 1, db = g.b_mn ? g.ldb0 : 1;   // the pairs share a stride
+  const int ra = g.a_mn ? 1 : g.lda0, rb = g.b_mn ? 1 : g.ldb0;
+  for (int o = threadIdx.x; o < total; o += SP_THREADS) {
+    const int m = o / N, n = o - m * N;
+    auto dot = [&](const void* A, const void* B, float acc) {
+      const float* a = static_cast<const float*>(A) + m * ra;
+      const float* b = static_cast<const float*>(B) + n * rb;
+#pragma unroll 8
+      for (int k = 0; k < K; ++k, a += da, b += db) acc = fmaf(*a, *b, acc);
+      return acc;
+    };
+    float acc0 = 0.f, acc1 = 0.f;
+    if (g.terms & T_C0_A0B0) acc0 = dot(g.A0, g.B0, acc0);
+    if (g.terms & T_C0_A1B0) acc0 = dot(g.A1, g.B0, acc0);
+    if (g.terms & T_C0_A0B1) acc0 = dot(g.A0, g.B1, acc0);
+    if (g.terms & T_C0_A1B1) acc0 = dot(g.A1, g.B1, acc0);
+    if (g.terms & T_C1_A1B0) acc1 = dot(g.A1, g.B0, acc1);
+    if (g.terms & T_C1_A0B1) acc1 = dot(g.A0, g.B1, acc1);
+    const EpiOut r = epi_eval(g.epi, m, n, acc0, acc1, g.bias0, g.bias1, dual);
+    if (g.C0) g.C0[m * g.ldc0 + n] = r.c0;
+    if (g.C1) g.C1[m * g.ldc1 + n] = r.c1;
+    if (g.epi.mode != EPI_STORE) {
+      if (g.epi.A) static_cast<float*>(g.epi.A)[m * g.epi.lda + n] = r.o0;
+      if (dual && g.epi.Ad) static_cast<float*>(g.epi.Ad)[m * g.epi.lda + n] = r.o1;
+    }
+  }
+}
+
+// Copy n bytes (a multiple of 16) of the kernel parameters or of global memory to or from
+// shared memory, 16 bytes per thread.  Through generic addresses: as indexed constant loads
+// the parameters would come one word at a time.
+__device__ __forceinline__ void copy16(void* dst, const void* src, int n) {
+  for (int o = threadIdx.x * 16; o < n; o += SP_THREADS * 16) {
+    uint4 v;
+    asm volatile("ld.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                 : "l"(static_cast<const char*>(src) + o));
+    *reinterpret_cast<uint4*>(static_cast<char*>(dst) + o) = v;
+  }
+}
+
+struct MovePtr {   // a pointer into the workspace -> the same place in its shared-memory image
+  char* base; char* image; int64_t bytes;
+  template <typename P>
+  __device__ __forceinline__ void operator()(P*& p) const {
+    char* q = reinterpret_cast<char*>(const_cast<void*>(static_cast<const void*>(p)));
+    if (q >= base && q < base + bytes) p = reinterpret_cast<P*>(image + (q - base));
+  }
+};
+
+__device__ __forceinline__ void move_op(SmallOp& op, const MovePtr& mv) {
+  switch (op.kind) {
+    case SMALL_GEMM: {
+      GemmArgs& g = *reinterpret_cast<GemmArgs*>(op.data);
+      mv(g.A0); mv(g.A1); mv(g.B0); mv(g.B1); mv(g.C0); mv(g.C1); mv(g.bias0); mv(g.bias1);
+      mv(g.epi.A); mv(g.epi.Ad); mv(g.epi.Z); mv(g.epi.Zd);
+      break;
+    }
+    case SMALL_LOSS: {
+      LossArgs& a = *reinterpret_cast<LossArgs*>(op.data);
+      mv(a.F); mv(a.Fd); mv(a.Yf); mv(a.Yi); mv(a.eta_w); mv(a.ex_w); mv(a.l); mv(a.ld);
+      mv(a.d_eta); mv(a.dF); mv(a.dFd);
+      break;
+    }
+    case SMALL_UPDATE: {
+      LayerUpdArgs& a = *reinterpret_cast<LayerUpdArgs*>(op.data);
+      mv(a.cast_src); mv(a.theta); mv(a.m); mv(a.g); mv(a.theta_out); mv(a.m_out); mv(a.theta_bar);
+      mv(a.Hu); mv(a.m_adj); mv(a.u_in); mv(a.u_out); mv(a.d_plr); mv(a.partials); mv(a.lr.plr);
+      mv(a.lr.slr); mv(a.v); mv(a.v_out); mv(a.v_adj); mv(a.m_prev); mv(a.mbar); mv(a.vbar);
+      break;
+    }
+    case SMALL_COPY: {
+      SmallCopy& c = *reinterpret_cast<SmallCopy*>(op.data);
+      mv(c.dst); mv(c.src);
+      break;
+    }
+    case SMALL_SUM: {
+      SmallSum& a = *reinterpret_cast<SmallSum*>(op.data);
+      mv(a.x); mv(a.out);
+      break;
+    }
+    default: {
+      SmallRor& a = *reinterpret_cast<SmallRor*>(op.data);
+      mv(a.x); mv(a.D1); mv(a.D2); mv(a.dA); mv(a.zpart); mv(a.out);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(SP_THREADS) small_program_kernel(
+    const __grid_constant__ SmallProgram prog) {
+  __shared__ float red[SP_THREADS / 32];
+  extern __shared__ __align__(256) char image[];   // the workspace, then the program
+  SmallProgram& sp = *reinterpret_cast<SmallProgram*>(image + prog.ws_bytes);
+  LayerTable& tab = sp.tab;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, grp = tid / UPD_THREADS;
+  const int n = prog.n;
+  copy16(&sp, &prog, static_cast<int>(offsetof(SmallProgram, op)) + n * static_cast<int>(sizeof(SmallOp)));
+  __syncthreads();
+  const MovePtr mv{static_cast<char*>(prog.ws), image, prog.ws_bytes};
+  if (tid < n) move_op(sp.op[tid], mv);
+  if (tid < tab.n) { mv(tab.W[tid]); mv(tab.U[tid]); }
+  pdl_entry();
+  if (prog.load) copy16(image, prog.ws, prog.ws_bytes);   // left there by the call's last program
+  __syncthreads();
+  for (int i = 0; i < n; ++i) {
+    const SmallOp& op = sp.op[i];
+    switch (op.kind) {
+      case SMALL_GEMM: small_gemm(*reinterpret_cast<const GemmArgs*>(op.data)); break;
+      case SMALL_LOSS: {
+        const LossArgs& a = *reinterpret_cast<const LossArgs*>(op.data);
+        for (int row = warp; row < a.rows; row += SP_THREADS / 32) loss_seed_row<float>(a, row, lane);
+        break;
+      }
+      case SMALL_UPDATE: {   // a group of UPD_THREADS threads per block of the update
+        const LayerUpdArgs& a = *reinterpret_cast<const LayerUpdArgs*>(op.data);
+        for (int b = grp; b < tab.tile0[tab.n]; b += SP_GROUPS)
+          layer_update_block<float>(tab, a, b, tid % UPD_THREADS, red + grp * (UPD_THREADS / 32),
+                                    [&] { asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(UPD_THREADS) : "memory"); });
+        break;
+      }
+      case SMALL_COPY: {   // rows x cols floats; a null source writes value
+        const SmallCopy& c = *reinterpret_cast<const SmallCopy*>(op.data);
+        for (int e = tid; e < c.rows * c.cols; e += SP_THREADS) {
+          const int r = e / c.cols, x = e % c.cols;
+          c.dst[r * c.ldd + x] = c.src ? c.src[r * c.lds + x] : c.value;
+        }
+        break;
+      }
+      case SMALL_SUM: {
+        const SmallSum& a = *reinterpret_cast<const SmallSum*>(op.data);
+        float v = 0.f;
+        for (int e = tid; e < a.n; e += SP_THREADS) v += a.x[e];
+        v = warp_sum(v);
+        if (lane == 0) red[warp] = v;
+        __syncthreads();
+        if (warp == 0) {
+          v = warp_sum(lane < SP_THREADS / 32 ? red[lane] : 0.f);
+          if (lane == 0) a.out[0] = v * a.scale;
+        }
+        break;
+      }
+      case SMALL_ROR_FWD: {
+        const SmallRor& a = *reinterpret_cast<const SmallRor*>(op.data);
+        for (int e = tid; e < a.rows * a.cols; e += SP_THREADS) {
+          const int at = e / a.cols * a.ld + e % a.cols;
+          a.zpart[e] = a.x[e] * a.D2[e] * a.dA[e];
+          a.out[at] = a.x[e] * a.D1[e];
+        }
+        break;
+      }
+      case SMALL_ROR_BWD: {
+        const SmallRor& a = *reinterpret_cast<const SmallRor*>(op.data);
+        for (int e = tid; e < a.rows * a.cols; e += SP_THREADS) {
+          const int at = e / a.cols * a.ld + e % a.cols;
+          a.out[at] = a.zpart[e] + a.x[e] * a.D1[e];
+        }
+        break;
+      }
+    }
+    __syncthreads();
+  }
+  if (prog.save) copy16(prog.ws, image, prog.ws_bytes);
+}
+
 }  // namespace
+
+cudaError_t small_program(const SmallProgram& prog, cudaStream_t s) {
+  if (prog.n == 0) return cudaSuccess;
+  static PerDeviceOnce attr_once;
+  const cudaError_t e = attr_once.run([](int&) {
+    return cudaFuncSetAttribute(small_program_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kSmallImage + static_cast<int>(sizeof(SmallProgram)));
+  });
+  if (e != cudaSuccess) return e;
+  return launch_k(small_program_kernel, dim3(1), dim3(SP_THREADS),
+                  prog.ws_bytes + sizeof(SmallProgram), s, prog);
+}
 
 template <typename T>
 void fill_cols(const ColFill& f, int rows, cudaStream_t s) {
@@ -577,13 +785,9 @@ void sum_scaled(const float* x, int n, float scale, float* out, cudaStream_t s) 
   launch_k(sum_scaled_kernel, dim3(1), dim3(1024), 0, s, x, n, scale, out);
 }
 
-template <typename T>
-void layer_update(const LayerTable& tab, const LayerUpdArgs& args, cudaStream_t s) {
-  const int blocks = tab.tile0[tab.n];
-  if (blocks <= 0) return;
-  // float4 access only when every vector the call touches is 16-byte aligned (caller
-  // pointers such as theta or eta + offset need not be)
-  LayerUpdArgs a = args;
+// float4 access only when every vector the call touches is 16-byte aligned (caller pointers
+// such as theta or eta + offset need not be)
+bool update_vec_ok(const LayerUpdArgs& a) {
   uintptr_t any = 0;
   for (const void* p : {static_cast<const void*>(a.cast_src), static_cast<const void*>(a.theta),
                         static_cast<const void*>(a.m), static_cast<const void*>(a.g),
@@ -596,7 +800,15 @@ void layer_update(const LayerTable& tab, const LayerUpdArgs& args, cudaStream_t 
                         static_cast<const void*>(a.m_prev), static_cast<const void*>(a.mbar),
                         static_cast<const void*>(a.vbar)})
     any |= reinterpret_cast<uintptr_t>(p);
-  a.vec_ok = (any & 15) == 0;
+  return (any & 15) == 0;
+}
+
+template <typename T>
+void layer_update(const LayerTable& tab, const LayerUpdArgs& args, cudaStream_t s) {
+  const int blocks = tab.tile0[tab.n];
+  if (blocks <= 0) return;
+  LayerUpdArgs a = args;
+  a.vec_ok = update_vec_ok(a);
   launch_k(layer_update_kernel<T>, dim3(blocks), dim3(UPD_THREADS), 0, s, tab, a);
 }
 
