@@ -115,11 +115,153 @@ __global__ void loss_seed_kernel(const LossArgs a) {
   if (row < a.rows) loss_seed_row<T>(a, row, threadIdx.x & 31);
 }
 
+// The same for wide rows, one block per row: a warp crossed a wide row in strided passes one
+// load at a time (512 rows x 4096, squared error: 75 us; one block per row with sixteen-byte
+// loads in flight: 7 us).  From 129 columns on, where both take the same time at few rows;
+// a 1000-way cross-entropy at 1000 rows takes its call from 56 to 30 us.
+constexpr int LB_THREADS = 256, kBlockLossCols = 128;
+
+// Sum (or maximum) over the block, in every thread.
+template <bool MAX>
+__device__ __forceinline__ float block_reduce(float v, float* red) {
+  v = MAX ? warp_max(v) : warp_sum(v);
+  __syncthreads();   // red may still be read
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  float r = red[0];
+#pragma unroll
+  for (int i = 1; i < LB_THREADS / 32; ++i) r = MAX ? fmaxf(r, red[i]) : r + red[i];
+  return r;
+}
+
+// n (1 or 4) consecutive floats of p at c
+template <int N>
+__device__ __forceinline__ void ldn(float (&x)[N], const float* p, int c) {
+  if constexpr (N == 4) {
+    const float4 t = *reinterpret_cast<const float4*>(p + c);
+    x[0] = t.x; x[1] = t.y; x[2] = t.z; x[3] = t.w;
+  } else {
+    x[0] = p[c];
+  }
+}
+template <typename T, int N>
+__device__ __forceinline__ void stn(T* p, int64_t c, const float (&x)[N]) {
+  if constexpr (N == 1) {
+    p[c] = to_t<T>(x[0]);
+  } else if constexpr (sizeof(T) == 2) {
+    __nv_bfloat162 lo = __floats2bfloat162_rn(x[0], x[1]), hi = __floats2bfloat162_rn(x[2], x[3]);
+    uint2 v;
+    v.x = *reinterpret_cast<uint32_t*>(&lo);
+    v.y = *reinterpret_cast<uint32_t*>(&hi);
+    *reinterpret_cast<uint2*>(p + c) = v;
+  } else {
+    *reinterpret_cast<float4*>(p + c) = make_float4(x[0], x[1], x[2], x[3]);
+  }
+}
+
+template <typename T, int N>
+__global__ void __launch_bounds__(LB_THREADS) loss_seed_block_kernel(const LossArgs a) {
+  pdl_entry();
+  __shared__ float red[LB_THREADS / 32];
+  const int row = blockIdx.x, C = a.cols;
+  const float* f = a.F + static_cast<int64_t>(row) * C;
+  const float* fd = a.Fd ? a.Fd + static_cast<int64_t>(row) * C : nullptr;
+  float w = 1.f, sg = 0.f;
+  if (a.ex_w) w = a.ex_w[row];
+  else if (a.eta_w) { sg = 1.f / (1.f + expf(-a.eta_w[row])); w = sg; }
+  const float scale = w * a.inv_norm;
+  T* dF = a.dF ? static_cast<T*>(a.dF) + static_cast<int64_t>(row) * a.ldo : nullptr;
+  T* dFd = fd && a.dFd ? static_cast<T*>(a.dFd) + static_cast<int64_t>(row) * a.ldo : nullptr;
+  const int c0 = threadIdx.x * N;
+  constexpr int STEP = LB_THREADS * N;
+  float l = 0.f, ld = 0.f;
+  if (a.loss == 0) {
+    const float* y = a.Yf + static_cast<int64_t>(row) * C;
+    const float invC = 1.f / static_cast<float>(C);
+    float s2 = 0.f, s1 = 0.f;
+#pragma unroll 4
+    for (int c = c0; c < C; c += STEP) {
+      float fv[N], yv[N], dv[N] = {}, o[N];
+      ldn(fv, f, c);
+      ldn(yv, y, c);
+      if (fd) ldn(dv, fd, c);
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        const float r = fv[j] - yv[j];
+        s2 += r * r;
+        s1 += r * dv[j];
+        o[j] = scale * r * invC;
+        dv[j] = scale * dv[j] * invC;
+      }
+      if (dF) stn<T, N>(dF, c, o);
+      if (dFd) stn<T, N>(dFd, c, dv);
+    }
+    l = 0.5f * block_reduce<false>(s2, red) * invC;
+    ld = block_reduce<false>(s1, red) * invC;
+  } else {
+    const int y = a.Yi[row];
+    if (y < 0 || y >= C) {
+      if (threadIdx.x == 0 && a.status) atomicMax(a.status, 1);
+      return;
+    }
+    float mx = -INFINITY, se = 0.f, pf = 0.f;
+#pragma unroll 4
+    for (int c = c0; c < C; c += STEP) {
+      float fv[N];
+      ldn(fv, f, c);
+#pragma unroll
+      for (int j = 0; j < N; ++j) mx = fmaxf(mx, fv[j]);
+    }
+    mx = block_reduce<true>(mx, red);
+#pragma unroll 4
+    for (int c = c0; c < C; c += STEP) {
+      float fv[N];
+      ldn(fv, f, c);
+#pragma unroll
+      for (int j = 0; j < N; ++j) se += expf(fv[j] - mx);
+    }
+    const float lse = mx + logf(block_reduce<false>(se, red));
+    if (fd) {
+#pragma unroll 4
+      for (int c = c0; c < C; c += STEP) {
+        float fv[N], dv[N];
+        ldn(fv, f, c);
+        ldn(dv, fd, c);
+#pragma unroll
+        for (int j = 0; j < N; ++j) pf += expf(fv[j] - lse) * dv[j];
+      }
+      pf = block_reduce<false>(pf, red);
+    }
+#pragma unroll 4
+    for (int c = c0; c < C; c += STEP) {
+      float fv[N], dv[N] = {}, o[N];
+      ldn(fv, f, c);
+      if (fd) ldn(dv, fd, c);
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        const float pc = expf(fv[j] - lse);
+        o[j] = scale * (pc - (c + j == y ? 1.f : 0.f));
+        dv[j] = scale * pc * (dv[j] - pf);
+      }
+      if (dF) stn<T, N>(dF, c, o);
+      if (dFd) stn<T, N>(dFd, c, dv);
+    }
+    l = lse - f[y];
+    if (fd) ld = pf - fd[y];
+  }
+  if (threadIdx.x == 0) {
+    if (a.l) a.l[row] = l;
+    if (a.ld) a.ld[row] = ld;
+    if (a.d_eta && a.eta_w) a.d_eta[row] = sg * (1.f - sg) * ld * a.inv_norm;
+  }
+}
+
 // Motivating example of Section 3 (Eq. 8): the model output is f = x theta followed by the
 // elementwise recursion y_0 = f, y_i = i (2 + sin y_{i-1})^cos y_{i-1}, i = 1..M, and
 // l_b = mean_o (y_M - t)^2.  Per element the recursion is carried with its first and second
 // derivatives in f (y', y''), so the loss seed 2/C r y' and its tangent 2/C (y'^2 + r y'') f'
 // come out of one pass; nothing of the recursion is stored.  One block per example.
+template <bool SECOND>
 __device__ __forceinline__ void chain_eval(float f, int M, float& y, float& d1, float& d2) {
   y = f; d1 = 1.f; d2 = 0.f;
   for (int i = 1; i <= M; ++i) {
@@ -128,58 +270,66 @@ __device__ __forceinline__ void chain_eval(float f, int M, float& y, float& d1, 
     const float b = 2.f + sn;                 // >= 1
     const float lb = logf(b);
     const float g1 = -sn * lb + cs * cs / b;  // d/dy [cos y log(2 + sin y)]
-    const float g2 = -cs * lb - 3.f * sn * cs / b - cs * cs * cs / (b * b);
     const float yi = static_cast<float>(i) * expf(cs * lb);
-    const float f1 = yi * g1, f2 = yi * (g1 * g1 + g2);
-    d2 = f2 * d1 * d1 + f1 * d2;
+    const float f1 = yi * g1;
+    if constexpr (SECOND) {
+      const float g2 = -cs * lb - 3.f * sn * cs / b - cs * cs * cs / (b * b);
+      d2 = yi * (g1 * g1 + g2) * d1 * d1 + f1 * d2;
+    }
     d1 = f1 * d1;
     y = yi;
   }
 }
 
-template <typename T>
-__global__ void chain_loss_kernel(const LossArgs a) {
+// Bound by the instructions of sincosf, logf, expf and the divisions of each step.  Without a
+// tangent the second derivatives are not formed: 1024 x 4096 at M = 3, primal 65 -> 39 us, dual
+// 53 us.
+template <typename T, bool DUAL, int N>
+__global__ void __launch_bounds__(LB_THREADS) chain_loss_kernel(const LossArgs a) {
   pdl_entry();
-  __shared__ float red[2][8];
+  __shared__ float red[LB_THREADS / 32];
   const int row = blockIdx.x;
   const int C = a.cols;
   const float* f = a.F + static_cast<int64_t>(row) * C;
-  const float* fd = a.Fd ? a.Fd + static_cast<int64_t>(row) * C : nullptr;
+  const float* fd = DUAL ? a.Fd + static_cast<int64_t>(row) * C : nullptr;
   const float* t = a.Yf + static_cast<int64_t>(row) * C;
   float w = 1.f, sg = 0.f;
   if (a.ex_w) w = a.ex_w[row];
   else if (a.eta_w) { sg = 1.f / (1.f + expf(-a.eta_w[row])); w = sg; }
   const float invC = 1.f / static_cast<float>(C);
   const float scale = w * a.inv_norm;
-  T* dF = static_cast<T*>(a.dF);
-  T* dFd = static_cast<T*>(a.dFd);
-  const int64_t orow = static_cast<int64_t>(row) * a.ldo;
+  T* dF = a.dF ? static_cast<T*>(a.dF) + static_cast<int64_t>(row) * a.ldo : nullptr;
+  T* dFd = DUAL && a.dFd ? static_cast<T*>(a.dFd) + static_cast<int64_t>(row) * a.ldo : nullptr;
   float s2 = 0.f, s1 = 0.f;
   bool bad = false;
-  for (int c = threadIdx.x; c < C; c += blockDim.x) {
-    float y, d1, d2;
-    chain_eval(f[c], a.chain, y, d1, d2);
-    const float r = y - t[c];
-    bad |= !isfinite(y) || !isfinite(d1);
-    s2 += r * r;
-    if (dF) dF[orow + c] = to_t<T>(scale * 2.f * invC * r * d1);
-    if (fd) {
-      const float ad = d1 * fd[c];
-      s1 += r * ad;
-      if (dFd) dFd[orow + c] = to_t<T>(scale * 2.f * invC * (d1 * ad + r * d2 * fd[c]));
+  for (int c = threadIdx.x * N; c < C; c += LB_THREADS * N) {
+    float fv[N], tv[N], dv[N] = {}, o[N], od[N];
+    ldn(fv, f, c);
+    ldn(tv, t, c);
+    if constexpr (DUAL) ldn(dv, fd, c);
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      float y, d1, d2;
+      chain_eval<DUAL>(fv[j], a.chain, y, d1, d2);
+      const float r = y - tv[j];
+      bad |= !isfinite(y) || !isfinite(d1);
+      s2 += r * r;
+      o[j] = scale * 2.f * invC * r * d1;
+      if constexpr (DUAL) {
+        const float ad = d1 * dv[j];
+        s1 += r * ad;
+        od[j] = scale * 2.f * invC * (d1 * ad + r * d2 * dv[j]);
+      }
+    }
+    if (dF) stn<T, N>(dF, c, o);
+    if constexpr (DUAL) {
+      if (dFd) stn<T, N>(dFd, c, od);
     }
   }
   if (bad && a.status) atomicMax(a.status, DEV_NONFINITE);
-  s2 = warp_sum(s2);
-  s1 = warp_sum(s1);
-  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (lane == 0) { red[0][wid] = s2; red[1][wid] = s1; }
-  __syncthreads();
+  const float l = block_reduce<false>(s2, red) * invC;
+  const float ld = DUAL ? block_reduce<false>(s1, red) * 2.f * invC : 0.f;
   if (threadIdx.x == 0) {
-    float l = 0.f, ld = 0.f;
-    for (int k = 0; k < static_cast<int>(blockDim.x >> 5); ++k) { l += red[0][k]; ld += red[1][k]; }
-    l *= invC;
-    ld *= 2.f * invC;
     if (a.l) a.l[row] = l;
     if (a.ld) a.ld[row] = ld;
     if (a.d_eta && a.eta_w) a.d_eta[row] = sg * (1.f - sg) * ld * a.inv_norm;
@@ -770,11 +920,25 @@ template <typename T>
 void loss_seed(const LossArgs& a, cudaStream_t s) {
   if (a.rows <= 0) return;
   if ((a.loss == 1 && !a.Yi) || (a.loss != 1 && !a.Yf) || !a.F) return;   // no targets: nothing read
+  // sixteen-byte access where every row is a multiple of it
+  auto al = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+  const bool vec = !(a.cols & 3) && !(a.ldo & 3) && al(a.F) && al(a.Fd) && al(a.Yf) && al(a.dF) && al(a.dFd);
+  const dim3 rows(a.rows), block(LB_THREADS);
   if (a.loss == 2) {
-    if (a.ror && a.tape && a.chain > 0 && (a.ror == 1 || a.Fd))
-      launch_k(chain_ror_kernel<T>, dim3(a.rows), dim3(256), 0, s, a);
-    else
-      launch_k(chain_loss_kernel<T>, dim3(a.rows), dim3(256), 0, s, a);
+    if (a.ror && a.tape && a.chain > 0 && (a.ror == 1 || a.Fd)) {
+      launch_k(chain_ror_kernel<T>, rows, dim3(256), 0, s, a);
+    } else if (a.Fd) {
+      if (vec) launch_k(chain_loss_kernel<T, true, 4>, rows, block, 0, s, a);
+      else launch_k(chain_loss_kernel<T, true, 1>, rows, block, 0, s, a);
+    } else {
+      if (vec) launch_k(chain_loss_kernel<T, false, 4>, rows, block, 0, s, a);
+      else launch_k(chain_loss_kernel<T, false, 1>, rows, block, 0, s, a);
+    }
+    return;
+  }
+  if (a.cols > kBlockLossCols) {
+    if (vec) launch_k(loss_seed_block_kernel<T, 4>, rows, block, 0, s, a);
+    else launch_k(loss_seed_block_kernel<T, 1>, rows, block, 0, s, a);
     return;
   }
   const int warps = 8;
