@@ -1199,8 +1199,11 @@ mf_status meta_grad_run(X& ex, const mf_loop_desc* lp, const float* theta0, cons
   auto m_at = [&](int t) { return ex.m_slot(st.m_idx(t)); };   // m_t, t >= 1
   const bool scalar_lr = lp->meta_kind & MF_META_SCALAR_LOGLR;
   ex.copy(theta_at(0), theta0, h->P);
-  const int64_t ne = n_eta_of(h, lp);
-  if (ne > 0) ex.zero(d_eta, ne);
+  const bool exw = lp->meta_kind & MF_META_EXAMPLE_WEIGHTS;
+  // the learning rates' part of d_eta is written by the first adjoint update and the final sum
+  if (exw) ex.zero(d_eta, static_cast<int64_t>(T) * B);
+  // without momentum u_t does not enter u_{t-1}, and Adam's never does
+  const bool u_carried = !st.adam && lp->momentum != 0.f;
   ex.prepare();
 
   // 1. rollout into the checkpoint store; the last segment stays in the segment slots
@@ -1242,7 +1245,9 @@ mf_status meta_grad_run(X& ex, const mf_loop_desc* lp, const float* theta0, cons
     a.m_adj = lr.lr_meta ? m_at(T) : nullptr;
     a.u_out = u;
     if (st.adam) adam_pre(a, T - 1, false);
+    a.u_copy = !u_carried;
     a.d_plr = d_plr;
+    a.plr_first = true;
     a.partials = scalar_lr ? part + static_cast<int64_t>(T - 1) * nb : nullptr;
     a.cast_src = theta_at(T - 1);
     a.mu = lp->momentum;
@@ -1254,7 +1259,6 @@ mf_status meta_grad_run(X& ex, const mf_loop_desc* lp, const float* theta0, cons
   // 3. reverse sweep
   const size_t xs = ex.x_step_bytes(B);
   const size_t ys = ex.y_step_bytes(B);
-  const bool exw = lp->meta_kind & MF_META_EXAMPLE_WEIGHTS;
   bool adam_pending = false;   // Adam's reverse of step t waits for its segment's recompute
   for (int t = T - 1; t >= 0; --t) {
     // entering an earlier segment [t+1-k, t+1): rebuild theta and m of its steps from the
@@ -1271,6 +1275,7 @@ mf_status meta_grad_run(X& ex, const mf_loop_desc* lp, const float* theta0, cons
       a.mode = mf::LU_ADJOINT;
       a.theta_bar = tbar;
       adam_pre(a, t, true);
+      a.u_copy = true;
       a.d_plr = d_plr;
       a.partials = scalar_lr ? part + static_cast<int64_t>(t) * nb : nullptr;
       a.lr = lr.lr;
@@ -1295,8 +1300,9 @@ mf_status meta_grad_run(X& ex, const mf_loop_desc* lp, const float* theta0, cons
       adam_pending = true;
     } else if (t > 0) {
       a.m_adj = lr.lr_meta ? m_at(t) : nullptr;
-      a.u_in = u;
+      a.u_in = u_carried ? u : nullptr;
       a.u_out = u;
+      a.u_copy = !u_carried;
       if (st.adam) adam_pre(a, t - 1, true);
       a.d_plr = d_plr;
       a.partials = scalar_lr ? part + static_cast<int64_t>(t - 1) * nb : nullptr;
@@ -1442,6 +1448,7 @@ mf_status meta_grad_run_binomial(X& ex, const mf_loop_desc* lp, const float* the
     pend_bar_in = bar_in;
     return MF_OK;
   };
+  const bool u_carried = !st.adam && lp->momentum != 0.f;   // as in meta_grad_run
   // u_{T-1} = -lr theta_bar_T ; d eta_lr += -lr m_T theta_bar_T ; cast theta_{T-1}, u_{T-1}
   {
     const int prev = next_rev(T);
@@ -1454,6 +1461,7 @@ mf_status meta_grad_run_binomial(X& ex, const mf_loop_desc* lp, const float* the
       a.theta_bar = tbar;
       a.m_adj = lr.lr_meta ? sl.m(ex, sT) : nullptr;
       a.u_out = u;
+      a.u_copy = !u_carried;
       if (st.adam) adam_pre(a, T - 1, false, sl.m(ex, sT), sl.v(ex, sT), prev);
       a.d_plr = d_plr;
       a.partials = scalar_lr ? part + static_cast<int64_t>(T - 1) * nb : nullptr;
@@ -1508,8 +1516,9 @@ mf_status meta_grad_run_binomial(X& ex, const mf_loop_desc* lp, const float* the
       defer = true;
     } else if (t > 0) {
       a.m_adj = lr.lr_meta ? sl.m(ex, cs) : nullptr;
-      a.u_in = u;
+      a.u_in = u_carried ? u : nullptr;
       a.u_out = u;
+      a.u_copy = !u_carried;
       if (st.adam) adam_pre(a, t - 1, true, sl.m(ex, cs), sl.v(ex, cs), prev);
       a.d_plr = d_plr;
       a.partials = scalar_lr ? part + static_cast<int64_t>(t - 1) * nb : nullptr;

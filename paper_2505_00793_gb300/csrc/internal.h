@@ -225,6 +225,10 @@ struct LayerUpdArgs {
   float* theta_bar = nullptr; const float* Hu = nullptr; const float* m_adj = nullptr;
   const float* u_in = nullptr; float* u_out = nullptr; float* d_plr = nullptr;
   float* partials = nullptr;       // scalar log-lr: one partial per block (tile)
+  bool plr_first = false;          // d_plr is written, not added to
+  // u' of a matrix element is read through its operand copy alone (no momentum carries u to
+  // the next step), so its float32 value is not written
+  bool u_copy = false;
   float mu = 0.f;
   LrArgs lr;
   int* status = nullptr;
