@@ -298,9 +298,9 @@ mf_status mf_replay_gemms(mf_handle h, int reps, void* stream, double* ms, uint6
  * MF_OPT_FLASH_ATTN (default 1): the decoder's dual attention runs fused, without the
  * S x S probabilities and their tangent in memory (bf16 decoders with d_model/n_heads = 64
  * and seq_len a multiple of 64; others always use the materialised form).  With 1, for
- * sequences of whole 128-token tiles, the dual (tangent-carrying) forward and both backward
- * kernels (primal and dual) run on tcgen05 tensor cores and the primal forward on
- * warp-level MMAs; 3 runs the primal forward on tcgen05 as well; 4 keeps the backward on
+ * sequences of whole 128-token tiles, the dual (tangent-carrying) forward, both backward
+ * kernels (primal and dual) and, from 256 tokens on, the primal forward run on tcgen05 tensor
+ * cores; 3 runs the primal forward of 128 tokens there as well; 4 keeps the backward on
  * warp-level MMAs; 2 uses the warp-level kernels only.  0 materialises them (per
  * block, for the backward).  Setting it drops the handle's captured graphs and changes the
  * workspace size.

@@ -4,16 +4,20 @@
 // the formulas, the D / D' prep and the warp-level kernels used for other lengths).
 //
 // Forward: one CTA per (head, 128-query tile), walking 64-key tiles up to the diagonal:
-//   warp 0      TMA producer: Q (and Q') once, then K, V (and K', V') per key tile into a
-//               ring of shared-memory stages (128-byte swizzle, K-major rows of 64 dims);
+//   warp 0      TMA producer: Q (and Q') once, then per key tile K (and K') into one ring of
+//               shared-memory stages and V (and V') into another (128-byte swizzle, K-major
+//               rows of 64 dims).  A K stage is free once its scores are computed, so even the
+//               dual kernel's single stages load the next K during this tile's softmax;
 //   warp 1      owns TMEM; one thread issues the MMAs:
 //                 S  = Q K^T,  S' = Q' K^T + Q K'^T            (M 128, N 64 keys, K 64)
 //                 O += P V,  T += (P (*) S') V + P V'          (M 128, N 64, K 64 keys; V
 //                                                               and V' read MN-major in place)
 //               with the products that share an A operand as one N = 128 MMA over adjacent
 //               B tiles and accumulators: Q [K | K']^T -> [S | Q K'^T], P [V | V'] -> [O | P V']
+//               and the next tile's scores are issued as soon as this tile's have been read;
 //   warps 2..5  softmax: thread r owns query row r (TMEM lane r).  It reads its row of S
-//               (and S') from TMEM, updates the running maximum, writes P = exp(S - m) and
+//               (and S') from TMEM, releases it, updates the running maximum, writes
+//               P = exp(S - m) and
 //               P (*) S' as bf16 into shared memory (the A operands of the next products) and
 //               keeps l = sum P and r = sum P (*) S'.
 // The tangent's two products share one accumulator T, since O' needs only their sum:
@@ -25,6 +29,13 @@
 // TAU = 8 (then O, T, l and r of the row are rescaled in place); between moves P may reach
 // e^8.  Every quantity of the row uses the same m, so O = o / l, the log-sum-exp
 // lse = m + log l, rbar = r / l and O' are exact for any m; only overflow needs the bound.
+//
+// What bounds it: shared memory, then the softmax warps' instructions.  A dual key tile moves
+// about 180 KB through shared memory (MMA operands, P, TMA), 1,400 of its 2,570 clocks an SM
+// at 128 bytes a clock; the elementwise arithmetic runs on float32 pairs with one multiply and
+// one exponential-unit instruction per e^x, and only the two tiles on the diagonal compare
+// positions.  128 heads of 1024 tokens: 142 -> 82 us dual, 91 -> 45 us primal (warp-level
+// MMAs 67 us), 128 heads of 256 tokens: 22 -> 14 and 14 -> 9 us.
 //
 // Every wait is bounded (2 s); a role that gives up records the timeout in the status word
 // and raises a CTA-local abort flag; the MMA thread then waits for its own last commit and
@@ -49,8 +60,8 @@ constexpr int BT_Q = 64;           // backward: queries (key-tile kernel) or key
 template <bool DUAL>
 struct FtcCfg {
   static constexpr int STAGES = DUAL ? 1 : 2;
-  static constexpr int STAGE_B = (DUAL ? 4 : 2) * K_TILE_B;  // K, (K',) V (, V')
-  static constexpr int OFF_V = (DUAL ? 2 : 1) * K_TILE_B;     // K' follows K, V' follows V
+  static constexpr int TILE_B = (DUAL ? 2 : 1) * K_TILE_B;    // K (, K'); V (, V')
+  static constexpr int STAGE_B = 2 * TILE_B;                 // K tiles, then V tiles
   static constexpr int Q_B = (DUAL ? 2 : 1) * Q_TILE_B;      // Q (Q')
   static constexpr int P_B = (DUAL ? 2 : 1) * P_ATOM;        // P (P (*) S')
   static constexpr int SMEM = Q_B + STAGES * STAGE_B + P_B + 1024;
@@ -104,6 +115,45 @@ __device__ __forceinline__ void tmem_wait_ld() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// Pairs of float32: sm_103a runs an operation on both halves as one instruction, each rounded
+// as the scalar operation is.
+__device__ __forceinline__ uint64_t pair(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 halves(uint64_t a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+// e^x of a pair as 2^(x log2 e) on the exponential unit (subnormal results become zero).
+__device__ __forceinline__ float2 exp_pair(uint64_t x) {
+  float2 t = halves(mul2(x, pair(1.44269504f, 1.44269504f)));
+  asm("ex2.approx.ftz.f32 %0, %0;" : "+f"(t.x));
+  asm("ex2.approx.ftz.f32 %0, %0;" : "+f"(t.y));
+  return t;
+}
+__device__ __forceinline__ uint32_t pack2(uint64_t a) {
+  const float2 v = halves(a);
+  return pack_bf16x2(v.x, v.y);
+}
+
 __device__ __forceinline__ void mbar_arrive_local(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
@@ -155,15 +205,17 @@ __global__ void __launch_bounds__(FTC_THREADS, FtcCfg<DUAL>::CTAS)
   const FtcParams p = prm;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   __shared__ __align__(8) uint64_t q_full, s_full, s_free, p_full, o_done, drain;
-  __shared__ __align__(8) uint64_t kv_full[C::STAGES], kv_empty[C::STAGES];
+  __shared__ __align__(8) uint64_t k_full[C::STAGES], k_empty[C::STAGES];
+  __shared__ __align__(8) uint64_t v_full[C::STAGES], v_empty[C::STAGES];
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
 
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   uint8_t* sQ = smem;                       // Q, then Q'
-  uint8_t* sKV = smem + C::Q_B;             // stage st: K, K', V, V' (8 KB each)
-  uint8_t* sP = sKV + C::STAGES * C::STAGE_B;   // P, then P (*) S' (16 KB each)
+  uint8_t* sK = smem + C::Q_B;              // stage st: K, K' (8 KB each)
+  uint8_t* sV = sK + C::STAGES * C::TILE_B; // stage st: V, V'
+  uint8_t* sP = sV + C::STAGES * C::TILE_B; // P, then P (*) S' (16 KB each)
   const int nq = p.S / TQ;
   // grid (heads, tiles): heads dispatch fastest, so every head's longest query tile goes
   // first and the shortest ones fill the tail of the launch
@@ -181,8 +233,10 @@ __global__ void __launch_bounds__(FTC_THREADS, FtcCfg<DUAL>::CTAS)
     mbar_init(&o_done, 1);
     mbar_init(&drain, 1);
     for (int i = 0; i < C::STAGES; ++i) {
-      mbar_init(&kv_full[i], 1);
-      mbar_init(&kv_empty[i], 1);
+      mbar_init(&k_full[i], 1);
+      mbar_init(&k_empty[i], 1);
+      mbar_init(&v_full[i], 1);
+      mbar_init(&v_empty[i], 1);
     }
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -214,24 +268,28 @@ __global__ void __launch_bounds__(FTC_THREADS, FtcCfg<DUAL>::CTAS)
       mbar_expect_tx(&q_full, C::Q_B);
       tma_load_3d(sQ, &tmQ, &q_full, 0, row0 + qt * TQ, 0);
       if (DUAL) tma_load_3d(sQ + Q_TILE_B, &tmQd, &q_full, 0, row0 + qt * TQ, 0);
-      int issued = 0;
-      for (int j = 0; j < nkt; ++j, ++issued) {
+      int nk = 0, nv = 0;
+      for (int j = 0; j < nkt; ++j) {
         const int st = j % C::STAGES;
-        const uint32_t ph = (j / C::STAGES) & 1;
-        if (!fwait(&kv_empty[st], ph ^ 1, p.status, abort)) break;
-        mbar_expect_tx(&kv_full[st], C::STAGE_B);
-        uint8_t* b = sKV + st * C::STAGE_B;
+        const uint32_t ph = ((j / C::STAGES) & 1) ^ 1;
         const int kr = row0 + j * TK;
-        tma_load_3d(b, &tmK, &kv_full[st], 0, kr, 0);
-        tma_load_3d(b + C::OFF_V, &tmV, &kv_full[st], 0, kr, 0);
-        if (DUAL) {
-          tma_load_3d(b + K_TILE_B, &tmKd, &kv_full[st], 0, kr, 0);
-          tma_load_3d(b + 3 * K_TILE_B, &tmVd, &kv_full[st], 0, kr, 0);
-        }
+        if (!fwait(&k_empty[st], ph, p.status, abort)) break;
+        mbar_expect_tx(&k_full[st], C::TILE_B);
+        uint8_t* b = sK + st * C::TILE_B;
+        tma_load_3d(b, &tmK, &k_full[st], 0, kr, 0);
+        if (DUAL) tma_load_3d(b + K_TILE_B, &tmKd, &k_full[st], 0, kr, 0);
+        ++nk;
+        if (!fwait(&v_empty[st], ph, p.status, abort)) break;
+        mbar_expect_tx(&v_full[st], C::TILE_B);
+        b = sV + st * C::TILE_B;
+        tma_load_3d(b, &tmV, &v_full[st], 0, kr, 0);
+        if (DUAL) tma_load_3d(b + K_TILE_B, &tmVd, &v_full[st], 0, kr, 0);
+        ++nv;
       }
       // every load issued has landed before the CTA can end
       mbar_wait(&q_full, 0, p.status, FTC_WAIT_NS);
-      drain_loads(kv_full, issued, C::STAGES, p.status);
+      drain_loads(k_full, nk, C::STAGES, p.status);
+      drain_loads(v_full, nv, C::STAGES, p.status);
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -244,16 +302,14 @@ __global__ void __launch_bounds__(FTC_THREADS, FtcCfg<DUAL>::CTAS)
       // operand descriptors, built once: a byte offset moves a descriptor by offset >> 4
       const uint64_t dQ = sdesc_sw128(smem_u32(sQ)), dQd = dQ + (Q_TILE_B >> 4);
       const uint64_t dP = sdesc_sw128(smem_u32(sP)), dPS = dP + (P_ATOM >> 4);
-      const uint64_t dKV = sdesc_sw128(smem_u32(sKV)), mKV = sdesc_mn_sw128(smem_u32(sKV));
-      constexpr uint64_t ST_STEP = C::STAGE_B >> 4, V_STEP = C::OFF_V >> 4;
-      bool ok = fwait(&q_full, 0, p.status, abort);
-      for (int j = 0; ok && j < nkt; ++j) {
+      const uint64_t dKs = sdesc_sw128(smem_u32(sK)), mVs = sdesc_mn_sw128(smem_u32(sV));
+      constexpr uint64_t ST_STEP = C::TILE_B >> 4;
+      // S (and S') of key tile j, once its K tiles are in
+      auto scores = [&](int j) -> bool {
         const int st = j % C::STAGES;
-        const uint32_t ph = (j / C::STAGES) & 1;
-        if (!fwait(&kv_full[st], ph, p.status, abort)) break;
-        if (j > 0 && !fwait(&s_free, (j - 1) & 1, p.status, abort)) break;
+        if (!fwait(&k_full[st], (j / C::STAGES) & 1, p.status, abort)) return false;
         tc_fence_after();
-        const uint64_t dK = dKV + st * ST_STEP, mV = mKV + st * ST_STEP + V_STEP;
+        const uint64_t dK = dKs + st * ST_STEP;
         if (DUAL) {
           // Q [K | K']^T -> [S | Q K'^T] in one N = 128 MMA (K' follows K), then Q' K^T into S'
 #pragma unroll
@@ -268,8 +324,19 @@ __global__ void __launch_bounds__(FTC_THREADS, FtcCfg<DUAL>::CTAS)
             mma_bf16(tb + C::C_S, dQ + 2 * kk, dK + 2 * kk, idS, kk > 0);
         }
         mma_commit(&s_full);
+        mma_commit(&k_empty[st]);
+        return true;
+      };
+      bool ok = fwait(&q_full, 0, p.status, abort) && scores(0);
+      for (int j = 0; ok && j < nkt; ++j) {
+        const int st = j % C::STAGES;
+        // the softmax warps have read the scores of tile j: the next tile's may overwrite
+        if (!fwait(&s_free, j & 1, p.status, abort)) break;
+        if (j + 1 < nkt && !scores(j + 1)) break;
         if (!fwait(&p_full, j & 1, p.status, abort)) break;
+        if (!fwait(&v_full[st], (j / C::STAGES) & 1, p.status, abort)) break;
         tc_fence_after();
+        const uint64_t mV = mVs + st * ST_STEP;
 #pragma unroll
         for (int kk = 0; kk < TK / 16; ++kk) {
           const uint64_t vb = mV + 128 * kk;
@@ -282,7 +349,7 @@ __global__ void __launch_bounds__(FTC_THREADS, FtcCfg<DUAL>::CTAS)
             mma_bf16(tb + C::C_O, dP + 2 * kk, vb, idO, acc);
           }
         }
-        mma_commit(&kv_empty[st]);
+        mma_commit(&v_empty[st]);
         mma_commit(&o_done);
       }
       // every MMA issued here has completed before TMEM is released
@@ -310,37 +377,49 @@ __global__ void __launch_bounds__(FTC_THREADS, FtcCfg<DUAL>::CTAS)
         tmem_ld32_nowait(tb + lo + C::C_SD + 32, sd + 32);
       }
       tmem_wait_ld();
-      float mx0 = -INFINITY, mx1 = -INFINITY;
-#pragma unroll
-      for (int i = 0; i < TK; i += 2) {
-        if (kbase + i <= r) mx0 = fmaxf(mx0, sv[i]);
-        if (kbase + i + 1 <= r) mx1 = fmaxf(mx1, sv[i + 1]);
-      }
-      const float mx = fmaxf(mx0, mx1);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive_local(&s_free);   // the next tile's scores may be computed
+      // only the two tiles on the diagonal have masked keys
+      const bool diag = kbase + TK > 0;
       float scale = 1.f;
-      if (mx > m + TAU) {
-        scale = __expf(m - mx);
-        m = mx;
-      }
       // P and P (*) S' of this tile, in registers
       uint32_t pk[TK / 2], psk[TK / 2];
-      float l0 = 0.f, l1 = 0.f, r0s = 0.f, r1s = 0.f;
+      uint64_t l2 = 0, r2 = 0;
+      auto softmax_tile = [&](auto masked) {
+        constexpr bool MASK = decltype(masked)::value;
+        float mx0 = -INFINITY, mx1 = -INFINITY;
 #pragma unroll
-      for (int i = 0; i < TK; i += 2) {
-        const float p0 = kbase + i > r ? 0.f : __expf(sv[i] - m);
-        const float p1 = kbase + i + 1 > r ? 0.f : __expf(sv[i + 1] - m);
-        l0 += p0;
-        l1 += p1;
-        pk[i / 2] = pack_bf16x2(p0, p1);
-        if (DUAL) {
-          const float s0 = p0 * sd[i], s1 = p1 * sd[i + 1];
-          r0s += s0;
-          r1s += s1;
-          psk[i / 2] = pack_bf16x2(s0, s1);
+        for (int i = 0; i < TK; i += 2) {
+          if (!MASK || kbase + i <= r) mx0 = fmaxf(mx0, sv[i]);
+          if (!MASK || kbase + i + 1 <= r) mx1 = fmaxf(mx1, sv[i + 1]);
         }
-      }
-      l = l * scale + (l0 + l1);
-      rs = rs * scale + (r0s + r1s);
+        const float mx = fmaxf(mx0, mx1);
+        if (mx > m + TAU) {
+          scale = __expf(m - mx);
+          m = mx;
+        }
+        const uint64_t nm = pair(-m, -m);
+#pragma unroll
+        for (int i = 0; i < TK; i += 2) {
+          float2 e = exp_pair(add2(pair(sv[i], sv[i + 1]), nm));
+          if (MASK && kbase + i > r) e.x = 0.f;
+          if (MASK && kbase + i + 1 > r) e.y = 0.f;
+          const uint64_t p2 = pair(e.x, e.y);
+          l2 = add2(l2, p2);
+          pk[i / 2] = pack_bf16x2(e.x, e.y);
+          if (DUAL) {
+            const uint64_t ps = mul2(p2, pair(sd[i], sd[i + 1]));
+            r2 = add2(r2, ps);
+            psk[i / 2] = pack2(ps);
+          }
+        }
+      };
+      if (diag) softmax_tile(std::true_type{});
+      else softmax_tile(std::false_type{});
+      const float2 lh = halves(l2), rh = halves(r2);
+      l = l * scale + (lh.x + lh.y);
+      rs = rs * scale + (rh.x + rh.y);
       if (j > 0) {
         // the products of tile j - 1 are done: O, T may be rescaled and P rewritten
         if (!wwait(&o_done, (j - 1) & 1, p.status, abort)) { ok = false; break; }
@@ -373,10 +452,7 @@ __global__ void __launch_bounds__(FTC_THREADS, FtcCfg<DUAL>::CTAS)
       tc_fence_before();
       fence_async_smem();
       __syncwarp();
-      if (lane == 0) {
-        mbar_arrive_local(&s_free);
-        mbar_arrive_local(&p_full);
-      }
+      if (lane == 0) mbar_arrive_local(&p_full);
     }
     // ---- outputs: O = o / l, lse, and O' = T / l - rbar O, rbar = r / l -----------------
     if (ok && wwait(&o_done, (nkt - 1) & 1, p.status, abort)) {
@@ -477,8 +553,10 @@ cudaError_t launch_ftc_fwd(const FlashArgs& a, cudaStream_t s) {
 // Two kernels, as the warp-level backward: one CTA per (head, 128-key tile) for dK, dV and
 // their tangents, one per (head, 128-query tile) for dQ and its tangent, so every sum keeps
 // a fixed order.  The key-tile kernel walks 64-query tiles from the diagonal on:
-//   warp 0      TMA producer: K, V (K', V') once; per query tile Q, dO (Q', dO') and the
-//               row statistics lse, D (rbar, D') into a two-stage ring;
+//   warp 0      TMA producer: K, V (K', V') once; per query tile Q, dO (Q', dO') into a ring
+//               of three stages (primal: two, with two CTAs an SM): a stage is free when its
+//               tile's products are done, and with two the load of the next tile waited for
+//               them;
 //   warp 1      one thread issues the MMAs (M 128 keys, N 64, K 64):
 //                 S^T = K Q^T,  S'^T = K' Q^T + K Q'^T,  dP^T = V dO^T,
 //                 dP'^T = V' dO^T + V dO'^T                          (scores, TMEM)
@@ -492,28 +570,38 @@ cudaError_t launch_ftc_fwd(const FlashArgs& a, cudaStream_t s) {
 //               dS^T = P^T (*) (dP^T - D), P'^T = P^T (*) (S'^T - rbar),
 //               dS'^T = P'^T (*) (dP^T - D) + P^T (*) (dP'^T - D'), kept as bf16 in
 //               registers, then written to shared memory (the A operands) once the previous
-//               tile's accumulating products have read it.
+//               tile's accumulating products have read it.  The row statistics lse, D (rbar,
+//               D') of the next tile pass through their registers into one of two slots.
 // The query-tile kernel is the same with the roles of queries and keys exchanged: Q, dO
 // (Q', dO') stay resident, K, V (K', V') stream per 64-key tile, and dQ += dS K,
-// dQ' += dS' K + dS K' (K read MN-major).
-constexpr int BW_EW = 8;                       // elementwise warps: two per TMEM lane quadrant,
-                                               // each on half of the tile's 64 columns
-constexpr int BW_THREADS = 64 + 32 * BW_EW;
+// dQ' += dS' K + dS K' (K read MN-major); its ring has four stages (primal: three).
+//
+// What bounds them: shared memory.  A dual tile moves about 350 KB (key-tile kernel: MMA
+// operands 224, A operands written 64, TMA 32, statistics 32) and 230 KB (query-tile kernel),
+// 2,800 of 3,600 and 1,800 of 2,150 clocks at 128 bytes a clock; sixteen elementwise warps
+// instead of eight changed nothing.  Both kernels, 128 heads of 1024 tokens: 358 -> 276 us
+// dual, 167 -> 131 us primal; of 256 tokens: 57 -> 42 and 31 -> 25 us.
 constexpr int ROWS128_B = 128 * HD * 2;        // 16 KB: [128][64] bf16
 constexpr int ROWS64_B = 64 * HD * 2;          // 8 KB: [64][64] bf16
 constexpr int OPND_B = 128 * 64 * 2;           // 16 KB: [128][64] bf16 A operand
 
 template <bool DUAL>
 struct KvCfg {
+  static constexpr int EW = DUAL ? 8 : 8;       // elementwise warps
+  static constexpr int THREADS = 64 + 32 * EW;
   static constexpr int NRES = DUAL ? 4 : 2;    // K, V (K', V'): 128 rows each
   static constexpr int NT = DUAL ? 4 : 2;      // Q, (Q',) dO (, dO') per query tile: 64 rows
   static constexpr int OFF_DO = DUAL ? 2 * ROWS64_B : ROWS64_B;   // Q' right after Q, dO' after dO
   static constexpr int NSTAT = DUAL ? 4 : 2;   // lse, D (rbar, D'): 64 floats each
-  static constexpr int STAGES = 2;
-  static constexpr int STAT_OFF = NT * ROWS64_B;
-  static constexpr int STAGE_B = STAT_OFF + 1024;
+  static constexpr int STAGES = DUAL ? 3 : 2;
+  static constexpr int STAGE_B = NT * ROWS64_B;
   static constexpr int NOP = DUAL ? 4 : 2;     // P^T, dS^T (P'^T, dS'^T)
-  static constexpr int SMEM = NRES * ROWS128_B + STAGES * STAGE_B + NOP * OPND_B + 1024;
+  static constexpr int STAT_B = NSTAT * BT_Q * 4;   // row statistics of one query tile
+  // the dual kernel's buffers leave no room to round the base up: it begins on a 1024-byte
+  // boundary (the declared alignment), which the kernel checks
+  static constexpr int SLACK = DUAL ? 0 : 1024;
+  static constexpr int SMEM =
+      NRES * ROWS128_B + STAGES * STAGE_B + NOP * OPND_B + 2 * STAT_B + SLACK;
   static constexpr int CTAS = DUAL ? 1 : 2;
   static constexpr uint32_t TMEM_COLS = DUAL ? 512 : 256;
   static constexpr uint32_t C_S = 0, C_SD = 64, C_DP = DUAL ? 128 : 64, C_DPD = 192;
@@ -523,10 +611,12 @@ struct KvCfg {
 
 template <bool DUAL>
 struct QCfg {
+  static constexpr int EW = DUAL ? 8 : 8;
+  static constexpr int THREADS = 64 + 32 * EW;
   static constexpr int NRES = DUAL ? 4 : 2;    // Q, dO (Q', dO'): 128 rows each
   static constexpr int NT = DUAL ? 4 : 2;      // K, (K',) V (, V') per key tile: 64 rows
   static constexpr int OFF_V = DUAL ? 2 * ROWS64_B : ROWS64_B;    // K' right after K, V' after V
-  static constexpr int STAGES = 2;
+  static constexpr int STAGES = DUAL ? 4 : 3;
   static constexpr int STAGE_B = NT * ROWS64_B;
   static constexpr int NOP = DUAL ? 2 : 1;     // dS (dS')
   static constexpr int SMEM = NRES * ROWS128_B + STAGES * STAGE_B + NOP * OPND_B + 1024;
@@ -548,16 +638,7 @@ struct FtbParams {
   float qscale;
 };
 
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes,
-                                          uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
-
-// Four 16-column TMEM loads in flight, then one wait.
+// One 16-column TMEM load without its wait, so that several are in flight.
 __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, float (&v)[16]) {
   uint32_t r[16];
   asm volatile(
@@ -571,11 +652,12 @@ __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, float (&v)[16])
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// Columns cb .. cb + 31 of a 128 x 64 float32 accumulator row (this thread's TMEM lane) to
+// Columns cb .. cb + CW - 1 of a 128 x 64 float32 accumulator row (this thread's TMEM lane) to
 // global memory.
+template <int CW>
 __device__ __forceinline__ void store_acc_row(uint32_t taddr, float* dst, int cb) {
 #pragma unroll 1
-  for (int c0 = cb; c0 < cb + 32; c0 += 16) {
+  for (int c0 = cb; c0 < cb + CW; c0 += 16) {
     float v[16];
     tmem_ld16(taddr + c0, v);
 #pragma unroll
@@ -584,61 +666,73 @@ __device__ __forceinline__ void store_acc_row(uint32_t taddr, float* dst, int cb
   }
 }
 
-// Columns cb .. cb + 31 of a 64-wide accumulator row (this thread's TMEM lane, row r of
-// the tile) as bf16 into a [128][64] staging tile (128-byte rows, 16-byte chunk c of row r at
-// position c ^ (r & 7)), with the inverse RoPE rotation of position pos when rot is set: the
-// first half's element j becomes (x_j cos_j + x_{j+32} sin_j) scale, the second half's
-// (x_{j+32} cos_j - x_j sin_j) scale (the partner half is read from the same TMEM lane).
-__device__ __forceinline__ void stage_merged_row(uint32_t taddr, int cb, bool rot, int pos,
-                                                 const float* rtab, float scale, uint8_t* buf,
-                                                 int r) {
-  const int pb = cb ^ 32;
-  const float sg = cb == 0 ? 1.f : -1.f;
-#pragma unroll 1
-  for (int c0 = 0; c0 < 32; c0 += 16) {
-    float x[16], y[16];
-    tmem_ld16_nowait(taddr + cb + c0, x);
-    if (rot) tmem_ld16_nowait(taddr + pb + c0, y);
-    tmem_wait_ld();
-    uint32_t pk[8];
-#pragma unroll
-    for (int e = 0; e < 16; e += 2) {
-      float o0 = x[e], o1 = x[e + 1];
-      if (rot) {
-        const float4 t = *reinterpret_cast<const float4*>(rtab + 2 * (pos * 32 + c0 + e));
-        o0 = (x[e] * t.x + sg * y[e] * t.y) * scale;
-        o1 = (x[e + 1] * t.z + sg * y[e + 1] * t.w) * scale;
-      }
-      pk[e / 2] = pack_bf16x2(o0, o1);
-    }
-    const int ch = (cb + c0) >> 3;
-    *reinterpret_cast<uint4*>(buf + r * 128 + (((ch) ^ (r & 7)) << 4)) =
-        make_uint4(pk[0], pk[1], pk[2], pk[3]);
-    *reinterpret_cast<uint4*>(buf + r * 128 + (((ch + 1) ^ (r & 7)) << 4)) =
-        make_uint4(pk[4], pk[5], pk[6], pk[7]);
-  }
-}
-
-// The elementwise warps' barrier (named barrier 1, BW_EW warps).
+// The elementwise warps' barrier (named barrier 1).
+template <int EW>
 __device__ __forceinline__ void ew_bar() {
-  asm volatile("bar.sync 1, %0;" ::"n"(BW_EW * 32) : "memory");
+  asm volatile("bar.sync 1, %0;" ::"n"(EW * 32) : "memory");
 }
 
-// A staged [128][64] bf16 tile to 128 rows of global memory (row i at row_base(i)), by the
-// elementwise threads (et = 0 .. BW_EW*32 - 1): eight consecutive threads write one row's
-// 128 bytes.
-template <class RowBase>
-__device__ __forceinline__ void staged_rows_out(const uint8_t* buf, int et, RowBase row_base) {
-#pragma unroll 1
-  for (int i = et; i < 128 * 8; i += BW_EW * 32) {
-    const int row = i >> 3, c = i & 7;
-    const uint4 v = *reinterpret_cast<const uint4*>(buf + row * 128 + ((c ^ (row & 7)) << 4));
-    *reinterpret_cast<uint4*>(row_base(row) + c * 8) = v;
+// Merged outputs in two steps.  First each thread puts its columns of an accumulator row
+// (TMEM lane, row r of the tile) into a float32 [128][64] staging tile: 256-byte rows,
+// 16-byte chunk c of row r at position c ^ (r & 7).
+constexpr int OUT_TILE_B = 128 * HD * 4;
+template <int CW>
+__device__ __forceinline__ void stage_row(uint32_t taddr, int cb, uint8_t* buf, int r) {
+  float x[CW];
+#pragma unroll
+  for (int c0 = 0; c0 < CW; c0 += 16)
+    tmem_ld16_nowait(taddr + cb + c0, *reinterpret_cast<float(*)[16]>(x + c0));
+  tmem_wait_ld();
+#pragma unroll
+  for (int e = 0; e < CW; e += 4)
+    *reinterpret_cast<float4*>(buf + r * 256 + ((((cb + e) >> 2) ^ (r & 7)) << 4)) =
+        make_float4(x[e], x[e + 1], x[e + 2], x[e + 3]);
+}
+// Then eight threads write each row as bf16, ROT with the inverse RoPE rotation: the first
+// half's element j becomes (x_j cos_j + x_{j+32} sin_j) scale, the second half's
+// (x_{j+32} cos_j - x_j sin_j) scale; with DUAL the tangent's tile, after the primal's, too.
+// Rows of the (cos, sin) table (rtab: the tile's first position) and of the output are read
+// and written whole: threads that each rotated their own row, reading its table row and the
+// partner columns from TMEM, took 13,600 clocks a dual key tile where this takes 7,500.
+template <int EW, bool DUAL, bool ROT, class RowBase>
+__device__ __forceinline__ void rows_out(const uint8_t* buf, const uint8_t* bufd, int et,
+                                         const float* rtab, float scale, RowBase row_off,
+                                         __nv_bfloat16* out, __nv_bfloat16* outd) {
+  const int k = et & 7, c = 2 * k;   // output elements 8 k .. 8 k + 7, float4 chunks c, c + 1
+  const float sg = k < 4 ? 1.f : -1.f;
+#pragma unroll
+  for (int i = et >> 3; i < 128; i += EW * 4) {
+    float4 t[4];
+    if (ROT) {
+      const float4* tr = reinterpret_cast<const float4*>(rtab + i * 64 + (k & 3) * 16);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) t[j] = tr[j];
+    }
+    const int64_t o = row_off(i) + k * 8;
+#pragma unroll
+    for (int w = 0; w < (DUAL ? 2 : 1); ++w) {
+      const uint8_t* row = (w ? bufd : buf) + i * 256;
+      uint32_t pk[4];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        float4 x = *reinterpret_cast<const float4*>(row + (((c + j) ^ (i & 7)) << 4));
+        if (ROT) {
+          const float4 y = *reinterpret_cast<const float4*>(row + ((((c ^ 8) + j) ^ (i & 7)) << 4));
+          x.x = (x.x * t[2 * j].x + sg * y.x * t[2 * j].y) * scale;
+          x.y = (x.y * t[2 * j].z + sg * y.y * t[2 * j].w) * scale;
+          x.z = (x.z * t[2 * j + 1].x + sg * y.z * t[2 * j + 1].y) * scale;
+          x.w = (x.w * t[2 * j + 1].z + sg * y.w * t[2 * j + 1].w) * scale;
+        }
+        pk[2 * j] = pack_bf16x2(x.x, x.y);
+        pk[2 * j + 1] = pack_bf16x2(x.z, x.w);
+      }
+      *reinterpret_cast<uint4*>((w ? outd : out) + o) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+    }
   }
 }
 
 template <bool DUAL>
-__global__ void __launch_bounds__(BW_THREADS, KvCfg<DUAL>::CTAS)
+__global__ void __launch_bounds__(KvCfg<DUAL>::THREADS, KvCfg<DUAL>::CTAS)
     flash_tc_bwd_kv_kernel(const __grid_constant__ CUtensorMap tmK,
                            const __grid_constant__ CUtensorMap tmV,
                            const __grid_constant__ CUtensorMap tmKd,
@@ -658,8 +752,13 @@ __global__ void __launch_bounds__(BW_THREADS, KvCfg<DUAL>::CTAS)
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   uint8_t* sRes = smem;                                  // K, V, K', V'
-  uint8_t* sSt = smem + C::NRES * ROWS128_B;             // stage: Q, dO, Q', dO', statistics
+  uint8_t* sSt = smem + C::NRES * ROWS128_B;             // stage: Q, dO, Q', dO'
   uint8_t* sOp = sSt + C::STAGES * C::STAGE_B;           // P^T, dS^T, P'^T, dS'^T
+  float* sStat = reinterpret_cast<float*>(sOp + C::NOP * OPND_B);   // two tiles' statistics
+  if (C::SLACK == 0 && smem != smem_raw) {   // the whole grid alike, before any barrier
+    if (threadIdx.x == 0 && p.status) atomicMax(p.status, DEV_TIMEOUT);
+    return;
+  }
   // grid (heads, key tiles): heads fastest, and key tile 0 meets the most query tiles
   const int kt = static_cast<int>(blockIdx.y);
   const int bh = static_cast<int>(blockIdx.x);
@@ -672,8 +771,8 @@ __global__ void __launch_bounds__(BW_THREADS, KvCfg<DUAL>::CTAS)
   if (threadIdx.x == 0) {
     mbar_init(&res_full, 1);
     mbar_init(&s_full, 1);
-    mbar_init(&s_free, BW_EW);
-    mbar_init(&p_full, BW_EW);
+    mbar_init(&s_free, C::EW);
+    mbar_init(&p_full, C::EW);
     mbar_init(&o_done, 1);
     mbar_init(&drain, 1);
     for (int i = 0; i < C::STAGES; ++i) {
@@ -721,18 +820,14 @@ __global__ void __launch_bounds__(BW_THREADS, KvCfg<DUAL>::CTAS)
         const int st = i % C::STAGES;
         const uint32_t ph = (i / C::STAGES) & 1;
         if (!fwait(&st_empty[st], ph ^ 1, p.status, abort)) break;
-        mbar_expect_tx(&st_full[st], C::NT * ROWS64_B + C::NSTAT * BT_Q * 4);
+        mbar_expect_tx(&st_full[st], C::STAGE_B);
         uint8_t* b = sSt + st * C::STAGE_B;
         const int qr = row0 + (j0 + i) * BT_Q;
         tma_load_3d(b, &tmQ, &st_full[st], 0, qr, 0);
         tma_load_3d(b + C::OFF_DO, &tmdO, &st_full[st], 0, qr, 0);
-        bulk_load(b + C::STAT_OFF, p.lse + qr, BT_Q * 4, &st_full[st]);
-        bulk_load(b + C::STAT_OFF + 256, p.D + qr, BT_Q * 4, &st_full[st]);
         if (DUAL) {
           tma_load_3d(b + ROWS64_B, &tmQd, &st_full[st], 0, qr, 0);
           tma_load_3d(b + 3 * ROWS64_B, &tmdOd, &st_full[st], 0, qr, 0);
-          bulk_load(b + C::STAT_OFF + 512, p.rbar + qr, BT_Q * 4, &st_full[st]);
-          bulk_load(b + C::STAT_OFF + 768, p.Dd + qr, BT_Q * 4, &st_full[st]);
         }
       }
       // every load issued has landed before the CTA can end
@@ -829,19 +924,34 @@ __global__ void __launch_bounds__(BW_THREADS, KvCfg<DUAL>::CTAS)
     // ---- elementwise: key row r (TMEM lane r), query columns cb .. cb + 31 -----------------
     const int q4 = warp & 3;
     const int r = q4 * 32 + lane;
-    const int cb = ((warp - 2) >> 2) * 32;
+    constexpr int CW = 256 / C::EW;   // columns of this warp
+    const int cb = ((warp - 2) >> 2) * CW;
     const uint32_t lo = static_cast<uint32_t>(q4 * 32) << 16;
     const int key = key0 + r;
+    const uint64_t neg1 = pair(-1.f, -1.f);
+    // row statistics lse, D (, rbar, D') of the query tiles: a thread carries one value of the
+    // next tile in a register and stores it with its share of this tile's operands, so that
+    // p_full of this tile announces it (and that nobody reads the slot's old values any more)
+    const int et = threadIdx.x - 64, arr = et >> 6;
+    const float* stat_src = (arr == 0 ? p.lse : arr == 1 ? p.D : arr == 2 ? p.rbar : p.Dd) +
+                            row0 + j0 * BT_Q + (et & 63);
+    const bool stat_on = et < C::NSTAT * BT_Q;
+    if (stat_on) sStat[et] = stat_src[0];
+    ew_bar<C::EW>();
     bool ok = true;
     for (int i = 0; i < ntile; ++i) {
+      const float stat_next = stat_on && i + 1 < ntile ? stat_src[(i + 1) * BT_Q] : 0.f;
+      if (i > 0 && !wwait(&p_full, (i - 1) & 1, p.status, abort)) { ok = false; break; }
       if (!wwait(&s_full, i & 1, p.status, abort)) { ok = false; break; }
       tc_fence_after();
-      const float4* stat = reinterpret_cast<const float4*>(
-          sSt + (i % C::STAGES) * C::STAGE_B + C::STAT_OFF);   // lse, D, rbar, D' (16 float4 each)
+      // lse, D, rbar, D' (16 float4 each)
+      const float4* stat =
+          reinterpret_cast<const float4*>(sStat + (i & 1) * C::NSTAT * BT_Q);
       const int qbase = (j0 + i) * BT_Q;
-      uint32_t pk[16], dsk[16], pdk[DUAL ? 16 : 1], dsdk[DUAL ? 16 : 1];
+      const bool diag = qbase < key0 + 128;   // the only tiles with masked pairs
+      uint32_t pk[CW / 2], dsk[CW / 2], pdk[DUAL ? CW / 2 : 1], dsdk[DUAL ? CW / 2 : 1];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
+      for (int h = 0; h < CW / 16; ++h) {
         const int c0 = cb + 16 * h;
         float sv[16], dp[16], sd[16], dpd[16];
         tmem_ld16_nowait(tb + lo + C::C_S + c0, sv);
@@ -851,50 +961,50 @@ __global__ void __launch_bounds__(BW_THREADS, KvCfg<DUAL>::CTAS)
           tmem_ld16_nowait(tb + lo + C::C_DPD + c0, dpd);
         }
         tmem_wait_ld();
-        if (h == 1) {
+        if (h == CW / 16 - 1) {
           // this tile's scores are read: the next tile's may be computed meanwhile
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive_local(&s_free);
         }
+        auto half_tile = [&](auto masked) {
+          constexpr bool MASK = decltype(masked)::value;
 #pragma unroll
-        for (int e = 0; e < 16; e += 4) {
-          const int c = c0 + e;
-          const float4 l4 = stat[c / 4], d4 = stat[16 + c / 4];
-          float4 rb4 = make_float4(0.f, 0.f, 0.f, 0.f), dd4 = rb4;
-          if (DUAL) { rb4 = stat[32 + c / 4]; dd4 = stat[48 + c / 4]; }
-          const float lv[4] = {l4.x, l4.y, l4.z, l4.w}, dv[4] = {d4.x, d4.y, d4.z, d4.w};
-          const float rv[4] = {rb4.x, rb4.y, rb4.z, rb4.w}, ddv[4] = {dd4.x, dd4.y, dd4.z, dd4.w};
-          float pv[4], dsv[4], pdv[4], dsdv[4];
+          for (int e = 0; e < 16; e += 4) {
+            const int c = c0 + e;
+            const float4 l4 = stat[c / 4], d4 = stat[16 + c / 4];
+            float4 rb4 = make_float4(0.f, 0.f, 0.f, 0.f), dd4 = rb4;
+            if (DUAL) { rb4 = stat[32 + c / 4]; dd4 = stat[48 + c / 4]; }
+            const uint64_t lv[2] = {pair(l4.x, l4.y), pair(l4.z, l4.w)};
+            const uint64_t dv[2] = {pair(d4.x, d4.y), pair(d4.z, d4.w)};
+            const uint64_t rv[2] = {pair(rb4.x, rb4.y), pair(rb4.z, rb4.w)};
+            const uint64_t ddv[2] = {pair(dd4.x, dd4.y), pair(dd4.z, dd4.w)};
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const float pp = qbase + c + u >= key ? __expf(sv[e + u] - lv[u]) : 0.f;
-            const float dpm = dp[e + u] - dv[u];
-            pv[u] = pp;
-            dsv[u] = pp * dpm;
-            if (DUAL) {
-              const float pd = pp * (sd[e + u] - rv[u]);
-              pdv[u] = pd;
-              dsdv[u] = pd * dpm + pp * (dpd[e + u] - ddv[u]);
+            for (int u = 0; u < 2; ++u) {
+              const int f = e + 2 * u, k = (16 * h + f) / 2;
+              float2 pe = exp_pair(fma2(lv[u], neg1, pair(sv[f], sv[f + 1])));
+              if (MASK && qbase + c0 + f < key) pe.x = 0.f;
+              if (MASK && qbase + c0 + f + 1 < key) pe.y = 0.f;
+              const uint64_t pp = pair(pe.x, pe.y);
+              const uint64_t dpm = fma2(dv[u], neg1, pair(dp[f], dp[f + 1]));
+              pk[k] = pack_bf16x2(pe.x, pe.y);
+              dsk[k] = pack2(mul2(pp, dpm));
+              if (DUAL) {
+                const uint64_t pd = mul2(pp, fma2(rv[u], neg1, pair(sd[f], sd[f + 1])));
+                const uint64_t y = fma2(ddv[u], neg1, pair(dpd[f], dpd[f + 1]));
+                pdk[k] = pack2(pd);
+                dsdk[k] = pack2(fma2(pd, dpm, mul2(pp, y)));
+              }
             }
           }
-          const int k = (16 * h + e) / 2;
-          pk[k] = pack_bf16x2(pv[0], pv[1]);
-          pk[k + 1] = pack_bf16x2(pv[2], pv[3]);
-          dsk[k] = pack_bf16x2(dsv[0], dsv[1]);
-          dsk[k + 1] = pack_bf16x2(dsv[2], dsv[3]);
-          if (DUAL) {
-            pdk[k] = pack_bf16x2(pdv[0], pdv[1]);
-            pdk[k + 1] = pack_bf16x2(pdv[2], pdv[3]);
-            dsdk[k] = pack_bf16x2(dsdv[0], dsdv[1]);
-            dsdk[k + 1] = pack_bf16x2(dsdv[2], dsdv[3]);
-          }
-        }
+        };
+        if (diag) half_tile(std::true_type{});
+        else half_tile(std::false_type{});
       }
       // the previous tile's accumulating products have read the A operands
       if (i > 0 && !wwait(&o_done, (i - 1) & 1, p.status, abort)) { ok = false; break; }
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
+      for (int j = 0; j < CW / 8; ++j) {
         const uint32_t o = swz(r, cb / 8 + j);
         *reinterpret_cast<uint4*>(sOp + o) = make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
         *reinterpret_cast<uint4*>(sOp + OPND_B + o) =
@@ -906,6 +1016,7 @@ __global__ void __launch_bounds__(BW_THREADS, KvCfg<DUAL>::CTAS)
               make_uint4(dsdk[4 * j], dsdk[4 * j + 1], dsdk[4 * j + 2], dsdk[4 * j + 3]);
         }
       }
+      if (stat_on) sStat[((i + 1) & 1) * C::NSTAT * BT_Q + et] = stat_next;
       fence_async_smem();
       tc_fence_before();
       __syncwarp();
@@ -916,40 +1027,36 @@ __global__ void __launch_bounds__(BW_THREADS, KvCfg<DUAL>::CTAS)
     if (have) tc_fence_after();
     if (p.dqkv) {
       // merged rows: token b*S + key, k part (rotated) and v part of head h, staged in the
-      // A-operand buffers (the last products have read them) and written row by row; every
+      // operand buffers (every load has landed and the last products have read them); every
       // elementwise thread meets the barrier, with or without a result (a timed-out call
       // reports its status and its outputs are void)
       if (have) {
-        stage_merged_row(tb + lo + C::C_DK, cb, true, key, p.rope, 1.f, sOp, r);
-        stage_merged_row(tb + lo + C::C_DV, cb, false, key, p.rope, 1.f, sOp + OPND_B, r);
+        stage_row<CW>(tb + lo + C::C_DK, cb, smem, r);
+        stage_row<CW>(tb + lo + C::C_DV, cb, smem + OUT_TILE_B, r);
         if (DUAL) {
-          stage_merged_row(tb + lo + C::C_DKD, cb, true, key, p.rope, 1.f, sOp + 2 * OPND_B, r);
-          stage_merged_row(tb + lo + C::C_DVD, cb, false, key, p.rope, 1.f, sOp + 3 * OPND_B, r);
+          stage_row<CW>(tb + lo + C::C_DKD, cb, smem + 2 * OUT_TILE_B, r);
+          stage_row<CW>(tb + lo + C::C_DVD, cb, smem + 3 * OUT_TILE_B, r);
         }
       }
-      ew_bar();
+      ew_bar<C::EW>();
       if (have) {
         const int hh = bh % p.H, bb = bh / p.H, dm = p.H * HD;
-        const int et = threadIdx.x - 64;
-        auto base = [&](__nv_bfloat16* out, int part) {
-          return [=](int i) {
-            return out + (static_cast<int64_t>(bb) * p.S + key0 + i) * p.ldq + part * dm + hh * HD;
-          };
+        const float* rt = p.rope + key0 * HD;
+        auto row = [&](int i) {
+          return (static_cast<int64_t>(bb) * p.S + key0 + i) * p.ldq + dm + hh * HD;
         };
-        staged_rows_out(sOp, et, base(p.dqkv, 1));
-        staged_rows_out(sOp + OPND_B, et, base(p.dqkv, 2));
-        if (DUAL) {
-          staged_rows_out(sOp + 2 * OPND_B, et, base(p.dqkvd, 1));
-          staged_rows_out(sOp + 3 * OPND_B, et, base(p.dqkvd, 2));
-        }
+        rows_out<C::EW, DUAL, true>(smem, smem + 2 * OUT_TILE_B, et, rt, 1.f, row, p.dqkv,
+                                    p.dqkvd);
+        rows_out<C::EW, DUAL, false>(smem + OUT_TILE_B, smem + 3 * OUT_TILE_B, et, rt, 1.f, row,
+                                     p.dqkv + dm, p.dqkvd + dm);
       }
     } else if (have) {
       const int64_t off = (static_cast<int64_t>(row0) + key) * HD;
-      store_acc_row(tb + lo + C::C_DV, p.dV + off, cb);
-      store_acc_row(tb + lo + C::C_DK, p.dK + off, cb);
+      store_acc_row<CW>(tb + lo + C::C_DV, p.dV + off, cb);
+      store_acc_row<CW>(tb + lo + C::C_DK, p.dK + off, cb);
       if (DUAL) {
-        store_acc_row(tb + lo + C::C_DVD, p.dVd + off, cb);
-        store_acc_row(tb + lo + C::C_DKD, p.dKd + off, cb);
+        store_acc_row<CW>(tb + lo + C::C_DVD, p.dVd + off, cb);
+        store_acc_row<CW>(tb + lo + C::C_DKD, p.dKd + off, cb);
       }
     }
     tc_fence_before();
@@ -963,7 +1070,7 @@ __global__ void __launch_bounds__(BW_THREADS, KvCfg<DUAL>::CTAS)
 }
 
 template <bool DUAL>
-__global__ void __launch_bounds__(BW_THREADS, QCfg<DUAL>::CTAS)
+__global__ void __launch_bounds__(QCfg<DUAL>::THREADS, QCfg<DUAL>::CTAS)
     flash_tc_bwd_q_kernel(const __grid_constant__ CUtensorMap tmQ,
                           const __grid_constant__ CUtensorMap tmdO,
                           const __grid_constant__ CUtensorMap tmQd,
@@ -997,8 +1104,8 @@ __global__ void __launch_bounds__(BW_THREADS, QCfg<DUAL>::CTAS)
   if (threadIdx.x == 0) {
     mbar_init(&res_full, 1);
     mbar_init(&s_full, 1);
-    mbar_init(&s_free, BW_EW);
-    mbar_init(&p_full, BW_EW);
+    mbar_init(&s_free, C::EW);
+    mbar_init(&p_full, C::EW);
     mbar_init(&o_done, 1);
     mbar_init(&drain, 1);
     for (int i = 0; i < C::STAGES; ++i) {
@@ -1138,20 +1245,24 @@ __global__ void __launch_bounds__(BW_THREADS, QCfg<DUAL>::CTAS)
     // ---- elementwise: query row r (TMEM lane r), key columns cb .. cb + 31 -----------------
     const int q4 = warp & 3;
     const int r = q4 * 32 + lane;
-    const int cb = ((warp - 2) >> 2) * 32;
+    constexpr int CW = 256 / C::EW;   // columns of this warp
+    const int cb = ((warp - 2) >> 2) * CW;
     const uint32_t lo = static_cast<uint32_t>(q4 * 32) << 16;
     const int q = q0 + r;
     const int64_t gi = static_cast<int64_t>(row0) + q;
     const float lse = p.lse[gi], Dv = p.D[gi];
     const float rb = DUAL ? p.rbar[gi] : 0.f, Ddv = DUAL ? p.Dd[gi] : 0.f;
+    const uint64_t nlse = pair(-lse, -lse), nD = pair(-Dv, -Dv);
+    const uint64_t nrb = pair(-rb, -rb), nDd = pair(-Ddv, -Ddv);
     bool ok = true;
     for (int i = 0; i < ntile; ++i) {
       if (!wwait(&s_full, i & 1, p.status, abort)) { ok = false; break; }
       tc_fence_after();
       const int kbase = i * BT_Q;
-      uint32_t dsk[16], dsdk[DUAL ? 16 : 1];
+      const bool diag = kbase + BT_Q > q0;   // the only tiles with masked pairs
+      uint32_t dsk[CW / 2], dsdk[DUAL ? CW / 2 : 1];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
+      for (int h = 0; h < CW / 16; ++h) {
         const int c0 = cb + 16 * h;
         float sv[16], dp[16], sd[16], dpd[16];
         tmem_ld16_nowait(tb + lo + C::C_S + c0, sv);
@@ -1161,32 +1272,35 @@ __global__ void __launch_bounds__(BW_THREADS, QCfg<DUAL>::CTAS)
           tmem_ld16_nowait(tb + lo + C::C_DPD + c0, dpd);
         }
         tmem_wait_ld();
-        if (h == 1) {
+        if (h == CW / 16 - 1) {
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive_local(&s_free);
         }
+        auto half_tile = [&](auto masked) {
+          constexpr bool MASK = decltype(masked)::value;
 #pragma unroll
-        for (int e = 0; e < 16; e += 2) {
-          float dsv[2], dsdv[2];
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const int key = kbase + c0 + e + u;
-            const float pp = key <= q ? __expf(sv[e + u] - lse) : 0.f;
-            const float dpm = dp[e + u] - Dv;
-            dsv[u] = pp * dpm;
+          for (int e = 0; e < 16; e += 2) {
+            const int key = kbase + c0 + e, k = (16 * h + e) / 2;
+            float2 pe = exp_pair(add2(pair(sv[e], sv[e + 1]), nlse));
+            if (MASK && key > q) pe.x = 0.f;
+            if (MASK && key + 1 > q) pe.y = 0.f;
+            const uint64_t pp = pair(pe.x, pe.y);
+            const uint64_t dpm = add2(pair(dp[e], dp[e + 1]), nD);
+            dsk[k] = pack2(mul2(pp, dpm));
             if (DUAL) {
-              const float pd = pp * (sd[e + u] - rb);
-              dsdv[u] = pd * dpm + pp * (dpd[e + u] - Ddv);
+              const uint64_t pd = mul2(pp, add2(pair(sd[e], sd[e + 1]), nrb));
+              const uint64_t y = add2(pair(dpd[e], dpd[e + 1]), nDd);
+              dsdk[k] = pack2(fma2(pd, dpm, mul2(pp, y)));
             }
           }
-          dsk[(16 * h + e) / 2] = pack_bf16x2(dsv[0], dsv[1]);
-          if (DUAL) dsdk[(16 * h + e) / 2] = pack_bf16x2(dsdv[0], dsdv[1]);
-        }
+        };
+        if (diag) half_tile(std::true_type{});
+        else half_tile(std::false_type{});
       }
       if (i > 0 && !wwait(&o_done, (i - 1) & 1, p.status, abort)) { ok = false; break; }
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
+      for (int j = 0; j < CW / 8; ++j) {
         const uint32_t o = swz(r, cb / 8 + j);
         *reinterpret_cast<uint4*>(sOp + o) =
             make_uint4(dsk[4 * j], dsk[4 * j + 1], dsk[4 * j + 2], dsk[4 * j + 3]);
@@ -1203,27 +1317,26 @@ __global__ void __launch_bounds__(BW_THREADS, QCfg<DUAL>::CTAS)
     if (have) tc_fence_after();
     if (p.dqkv) {
       // merged rows: token b*S + q, q part (rotated and scaled) of head h, staged in the
-      // A-operand buffers and written row by row (every elementwise thread meets the barrier)
+      // operand buffers and written row by row (every elementwise thread meets the barrier)
       if (have) {
-        stage_merged_row(tb + lo + C::C_DQ, cb, true, q, p.rope, p.qscale, sOp, r);
-        if (DUAL) stage_merged_row(tb + lo + C::C_DQD, cb, true, q, p.rope, p.qscale, sOp + OPND_B, r);
+        stage_row<CW>(tb + lo + C::C_DQ, cb, smem, r);
+        if (DUAL) stage_row<CW>(tb + lo + C::C_DQD, cb, smem + OUT_TILE_B, r);
       }
-      ew_bar();
+      ew_bar<C::EW>();
       if (have) {
         const int hh = bh % p.H, bb = bh / p.H;
         const int et = threadIdx.x - 64;
-        auto base = [&](__nv_bfloat16* out) {
-          return [=](int i) {
-            return out + (static_cast<int64_t>(bb) * p.S + q0 + i) * p.ldq + hh * HD;
-          };
+        const float* rt = p.rope + q0 * HD;
+        auto row = [&](int i) {
+          return (static_cast<int64_t>(bb) * p.S + q0 + i) * p.ldq + hh * HD;
         };
-        staged_rows_out(sOp, et, base(p.dqkv));
-        if (DUAL) staged_rows_out(sOp + OPND_B, et, base(p.dqkvd));
+        rows_out<C::EW, DUAL, true>(smem, smem + OUT_TILE_B, et, rt, p.qscale, row, p.dqkv,
+                                    p.dqkvd);
       }
     } else if (have) {
       const int64_t off = gi * HD;
-      store_acc_row(tb + lo + C::C_DQ, p.dQ + off, cb);
-      if (DUAL) store_acc_row(tb + lo + C::C_DQD, p.dQd + off, cb);
+      store_acc_row<CW>(tb + lo + C::C_DQ, p.dQ + off, cb);
+      if (DUAL) store_acc_row<CW>(tb + lo + C::C_DQD, p.dQd + off, cb);
     }
     tc_fence_before();
   }
@@ -1278,10 +1391,10 @@ cudaError_t launch_ftc_bwd(const FlashArgs& a, cudaStream_t s) {
   p.rope = a.rope;
   p.qscale = a.qscale;
   const dim3 grid(a.BH, a.S / 128);
-  e = launch_k(flash_tc_bwd_kv_kernel<DUAL>, grid, dim3(BW_THREADS), KC::SMEM, s, k128[0],
+  e = launch_k(flash_tc_bwd_kv_kernel<DUAL>, grid, dim3(KC::THREADS), KC::SMEM, s, k128[0],
                k128[1], k128[2], k128[3], q64[0], q64[1], q64[2], q64[3], p);
   if (e != cudaSuccess) return e;
-  return launch_k(flash_tc_bwd_q_kernel<DUAL>, grid, dim3(BW_THREADS), QC::SMEM, s, q128[0],
+  return launch_k(flash_tc_bwd_q_kernel<DUAL>, grid, dim3(QC::THREADS), QC::SMEM, s, q128[0],
                   q128[1], q128[2], q128[3], k64[0], k64[1], k64[2], k64[3], p);
 }
 
