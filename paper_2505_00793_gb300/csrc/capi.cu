@@ -96,6 +96,7 @@ struct mf_ctx {
   // to the data product; ev_w[j] marks the end of the latest weight product that reads seed
   // buffer j, which the working stream waits for before it rewrites that buffer.
   cudaEvent_t ev_w[4] = {nullptr, nullptr, nullptr, nullptr};
+  cudaEvent_t ev_csr = nullptr;   // the backward's token lists, built on the side stream
   bool concurrent = true;
   int flash = 1;              // fused dual attention where supported (MF_OPT_FLASH_ATTN)
   // Per-layer parameter updates (MF_OPT_LAYER_UPDATES): an update stream that takes each
@@ -1649,8 +1650,9 @@ void destroy_handle_objects(mf_ctx* h) {
   if (h->sstream) cudaStreamDestroy(h->sstream);
   if (h->ustream) cudaStreamDestroy(h->ustream);
   for (cudaEvent_t e : {h->ev_in, h->ev_out, h->ev_fork, h->ev_join, h->ev_u_in, h->ev_u_out,
-                        h->ev_w[0], h->ev_w[1], h->ev_w[2], h->ev_w[3]})
+                        h->ev_w[0], h->ev_w[1], h->ev_w[2], h->ev_w[3], h->ev_csr})
     if (e) cudaEventDestroy(e);
+  h->ev_csr = nullptr;
   for (cudaEvent_t& e : h->ev_w) e = nullptr;
   h->d_status = nullptr;
   h->gstream = h->sstream = h->ustream = nullptr;
@@ -1737,6 +1739,7 @@ mf_status mf_create(const mf_model_desc* d, mf_handle* out) {
       cudaStreamCreateWithFlags(&h->ustream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_u_in, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_u_out, cudaEventDisableTiming) != cudaSuccess ||
+      cudaEventCreateWithFlags(&h->ev_csr, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_w[0], cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_w[1], cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_w[2], cudaEventDisableTiming) != cudaSuccess ||

@@ -496,8 +496,8 @@ struct DecExec {
   bool w_rec[4] = {false, false, false, false};
   bool side_used = false;
   bool conc() const {
-    return h->concurrent && h->sstream && h->ev_fork && h->ev_join && h->ev_w[0] &&
-           h->ev_w[1] && h->ev_w[2] && h->ev_w[3];
+    return h->concurrent && h->sstream && h->ev_fork && h->ev_join && h->ev_csr &&
+           h->ev_w[0] && h->ev_w[1] && h->ev_w[2] && h->ev_w[3];
   }
   void chk_cuda(cudaError_t e, const char* what) {
     if (e != cudaSuccess && st == MF_OK) {
@@ -558,6 +558,35 @@ struct DecExec {
     }
   }
 
+  // Backward of one RMSNorm into the residual gradient (and its operand-type seed dy), and the
+  // gain gradient's final sum.  The sum reads what the norm has just written and nothing on the
+  // working stream reads it, so it goes to the side stream: there it costs no time while the
+  // data products run (gpart is free again when the norm after this one waits for the seed's
+  // readers, which were queued behind it).
+  void norm_bwd(int rows, bool dual, const float* x, const float* xd, const float* r,
+                const float* rd, int64_t g, float* out_h, float* out_g, bool add, bool seed) {
+    const int N = rows * Ly.S, d = Ly.d;
+    wait_seed_readers(0);
+    float* part = at<float>(p.gpart);
+    const bool gain = out_g || dual;
+    const int nchunk = mf::dec_rmsnorm_bwd<T>(
+        N, d, x, xd, r, rd, theta_cur + g, dual ? u_cur + g : nullptr, at<float>(p.dh),
+        dual ? at<float>(p.dhd) : nullptr, at<float>(p.dx), at<float>(p.dxd), add, gain, part, s,
+        seed ? at<T>(p.dy) : nullptr, seed && dual ? at<T>(p.dyd) : nullptr);
+    launched();
+    if (!gain) return;
+    cudaStream_t q = s;
+    if (conc()) {
+      chk_cuda(cudaEventRecord(h->ev_fork, s), "side fork");
+      chk_cuda(cudaStreamWaitEvent(h->sstream, h->ev_fork, 0), "side fork");
+      q = h->sstream;
+      side_used = true;
+    }
+    mf::dec_gain_final(nchunk, d, dual, part, out_g ? out_g + g : nullptr,
+                       dual ? out_h + g : nullptr, q);
+    launched();
+  }
+
   // residual gradient (float32) -> operand-type seed
   // bf16 seeds dy (dy') of the next products from the residual-stream gradient dx (dx');
   // skipped when the RMSNorm backward that produced dx already wrote them (fresh)
@@ -577,12 +606,20 @@ struct DecExec {
     const int S = Ly.S, d = Ly.d, H = Ly.H, dh = Ly.dh, F = Ly.F, V = Ly.V;
     const int N = rows * S, BH = rows * H;
     const int64_t hs = static_cast<int64_t>(S) * dh, ss = static_cast<int64_t>(S) * S;
-    const float* u = u_cur;
     auto G = [&](int64_t off) { return out_g ? out_g + off : nullptr; };
     auto Hh = [&](int64_t off) { return dual ? out_h + off : nullptr; };
+    // the embedding gradient's token lists, next to the head's products (the weight products
+    // that follow on the side stream queue behind them)
+    const bool side = conc();
+    if (side) {
+      chk_cuda(cudaEventRecord(h->ev_fork, s), "side fork");
+      chk_cuda(cudaStreamWaitEvent(h->sstream, h->ev_fork, 0), "side fork");
+      side_used = true;
+    }
     mf::dec_token_csr(N, S, V, ids_cur, at<int>(p.o_count), at<int>(p.o_start), at<int>(p.o_order),
-                      at<int>(p.o_order_tmp), s);
+                      at<int>(p.o_order_tmp), side ? h->sstream : s);
     launched(4);
+    if (side) chk_cuda(cudaEventRecord(h->ev_csr, h->sstream), "token lists");
     // head: dWh = hf^T dF ; dhf = dF Wh^T
     wprod(d, V, at<T>(p.hf), at<T>(p.hfd), at<T>(p.dF), at<T>(p.dFd), dual, G(Ly.Wh), Hh(Ly.Wh));
     {
@@ -591,15 +628,8 @@ struct DecExec {
       g.C1 = at<float>(p.dhd); g.ldc1 = d;
       gemm(g);
     }
-    cudaMemsetAsync(at<float>(p.dx), 0, static_cast<size_t>(N) * d * 4, s);
-    if (dual) cudaMemsetAsync(at<float>(p.dxd), 0, static_cast<size_t>(N) * d * 4, s);
-    wait_seed_readers(0);
-    launched(mf::dec_rmsnorm_bwd<T>(N, d, at<float>(p.xf), at<float>(p.xfd), at<float>(p.rf),
-                                    at<float>(p.rfd), theta_cur + Ly.gf, dual ? u + Ly.gf : nullptr,
-                                    at<float>(p.dh), dual ? at<float>(p.dhd) : nullptr,
-                                    at<float>(p.dx), at<float>(p.dxd), G(Ly.gf), Hh(Ly.gf),
-                                    at<float>(p.gpart), s, at<T>(p.dy),
-                                    dual ? at<T>(p.dyd) : nullptr));
+    norm_bwd(rows, dual, at<float>(p.xf), at<float>(p.xfd), at<float>(p.rf), at<float>(p.rfd),
+             Ly.gf, out_h, out_g, false, true);
     for (int l = Ly.L - 1; l >= 0; --l) {
       if (ror_mode == 1) {
         cudaMemcpyAsync(at<float>(p.dxs[l]), at<float>(p.dx), static_cast<size_t>(N) * d * 4,
@@ -633,14 +663,8 @@ struct DecExec {
         g.C1 = at<float>(p.dhd); g.ldc1 = d;
         gemm(g);
       }
-      wait_seed_readers(0);
-      launched(mf::dec_rmsnorm_bwd<T>(N, d, at<float>(p.x2[l]), at<float>(p.x2d[l]),
-                                      at<float>(p.r2[l]), at<float>(p.r2d[l]), theta_cur + Ly.g2[l],
-                                      dual ? u + Ly.g2[l] : nullptr, at<float>(p.dh),
-                                      dual ? at<float>(p.dhd) : nullptr, at<float>(p.dx),
-                                      at<float>(p.dxd), G(Ly.g2[l]), Hh(Ly.g2[l]),
-                                      at<float>(p.gpart), s, at<T>(p.dy),
-                                      dual ? at<T>(p.dyd) : nullptr));
+      norm_bwd(rows, dual, at<float>(p.x2[l]), at<float>(p.x2d[l]), at<float>(p.r2[l]),
+               at<float>(p.r2d[l]), Ly.g2[l], out_h, out_g, true, true);
       // ---- attention branch: seed = dx (written in bf16 by the norm backward above) -----
       seed_from(at<float>(p.dx), at<float>(p.dxd), dual, true);
       wprod(d, d, at<T>(p.Om[l]), at<T>(p.Omd[l]), at<T>(p.dy), at<T>(p.dyd), dual, G(Ly.Wo[l]),
@@ -751,15 +775,10 @@ struct DecExec {
         g.C1 = at<float>(p.dhd); g.ldc1 = d;
         gemm(g);
       }
-      if (l > 0) wait_seed_readers(0);
-      launched(mf::dec_rmsnorm_bwd<T>(N, d, at<float>(p.x1[l]), at<float>(p.x1d[l]),
-                                      at<float>(p.r1[l]), at<float>(p.r1d[l]), theta_cur + Ly.g1[l],
-                                      dual ? u + Ly.g1[l] : nullptr, at<float>(p.dh),
-                                      dual ? at<float>(p.dhd) : nullptr, at<float>(p.dx),
-                                      at<float>(p.dxd), G(Ly.g1[l]), Hh(Ly.g1[l]),
-                                      at<float>(p.gpart), s, l > 0 ? at<T>(p.dy) : nullptr,
-                                      l > 0 && dual ? at<T>(p.dyd) : nullptr));
+      norm_bwd(rows, dual, at<float>(p.x1[l]), at<float>(p.x1d[l]), at<float>(p.r1[l]),
+               at<float>(p.r1d[l]), Ly.g1[l], out_h, out_g, true, l > 0);
     }
+    if (side) chk_cuda(cudaStreamWaitEvent(s, h->ev_csr, 0), "token lists");
     mf::dec_embed_bwd(V, d, at<int>(p.o_start), at<int>(p.o_order), at<float>(p.dx),
                       dual ? at<float>(p.dxd) : nullptr, G(Ly.E), Hh(Ly.E), s);
     launched();
