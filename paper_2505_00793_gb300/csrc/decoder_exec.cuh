@@ -362,18 +362,14 @@ struct DecExec {
         gemm(g);
       }
       const float qscale = 1.f / sqrtf(static_cast<float>(dh));
-      mf::dec_rope_split<T>(N, S, H, dh, at<float>(p.rope), qscale, at<float>(p.qkv), at<T>(p.Q[l]),
-                            at<T>(p.K[l]), at<T>(p.Vv[l]), s);
+      mf::RopeSplit<T> rs{at<float>(p.qkv), at<T>(p.Q[l]), at<T>(p.K[l]), at<T>(p.Vv[l])}, rsd;
+      if (dual) rsd = {at<float>(p.qkvd), at<T>(p.Qd[l]), at<T>(p.Kd[l]), at<T>(p.Vd[l])};
+      mf::dec_rope_split<T>(N, S, H, dh, at<float>(p.rope), qscale, rs, rsd, s);
       launched();
-      if (dual) {
-        mf::dec_rope_split<T>(N, S, H, dh, at<float>(p.rope), qscale, at<float>(p.qkvd), at<T>(p.Qd[l]),
-                              at<T>(p.Kd[l]), at<T>(p.Vd[l]), s);
-        launched();
-      }
 
       if (p.flash) {
-        // fused causal attention and its tangent: O, O' and the row statistics
-        // fused causal attention and its tangent, written head-merged as the Wo operands
+        // fused causal attention and its tangent: row statistics, and O, O' written head-merged
+        // as the Wo operands
         mf::FlashArgs fa = flash_args(l, BH);
         fa.H = H;
         fa.ldo = d;

@@ -127,7 +127,9 @@ __global__ void rmsnorm_fwd_kernel(int d, float eps, const float* __restrict__ x
 //   dx' += r' (dn - n c) + r (dn' - n' c - n c'),  dn' = dy' g + dy g',  c' = mean(dn' n + dn n')
 // Warp-per-row versions of the RMSNorm forward and backward (eight rows per block, float4
 // access, shuffle reductions), used when every vector is 16-byte aligned and d is a multiple
-// of 4; same arithmetic as the block-per-row kernels above and below.
+// of 4; same arithmetic as the block-per-row kernels above and below.  The forward
+// with NC > 0 loads rows of up to 128 NC columns once into registers, all loads in flight
+// together; with NC = 0 it walks them 128 columns at a time and reads them a second time.
 __device__ __forceinline__ float warp_sum_all(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -149,7 +151,20 @@ __device__ __forceinline__ void st_t4(T* p, float a, float b, float c, float d) 
 
 __device__ __forceinline__ float4 ld4f(const float* p) { return *reinterpret_cast<const float4*>(p); }
 
-template <typename T>
+// Columns 128 k + 4 lane .. + 3 of a row, for the k of this lane: a compile-time count when the
+// row is kept in registers.
+template <int NC, class F>
+__device__ __forceinline__ void row_quads(int d, int lane, F&& f) {
+  if constexpr (NC > 0) {
+#pragma unroll
+    for (int k = 0; k < NC; ++k)
+      if (k * 128 + lane * 4 < d) f(k, k * 128 + lane * 4);
+  } else {
+    for (int c = lane * 4; c < d; c += 128) f(0, c);
+  }
+}
+
+template <typename T, bool DUAL, int NC>
 __global__ void __launch_bounds__(256) rmsnorm_fwd_warp_kernel(
     int N, int d, float eps, const float* __restrict__ x_in, const float* __restrict__ y,
     const float* __restrict__ xd_in, const float* __restrict__ yd, const float* __restrict__ g,
@@ -157,23 +172,34 @@ __global__ void __launch_bounds__(256) rmsnorm_fwd_warp_kernel(
     float* __restrict__ rr, float* __restrict__ rrd, T* __restrict__ h, T* __restrict__ hd,
     int ldh) {
   pdl_entry();
+  constexpr int NK = NC > 0 ? NC : 1;
   const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (r >= N) return;
   const int64_t o = static_cast<int64_t>(r) * d;
-  const bool dual = xd_in != nullptr;
-  float s2 = 0.f, s1 = 0.f;
-  for (int c = lane * 4; c < d; c += 128) {
+  float4 xs[NK], xds[DUAL ? NK : 1];
+  auto load = [&](int k, int c) {
     float4 v = ld4f(x_in + o + c);
     if (y) { const float4 t = ld4f(y + o + c); v.x += t.x; v.y += t.y; v.z += t.z; v.w += t.w; }
-    *reinterpret_cast<float4*>(x_out + o + c) = v;
-    s2 += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
-    if (dual) {
+    xs[k] = v;
+    if constexpr (DUAL) {
       float4 vd = ld4f(xd_in + o + c);
       if (yd) { const float4 t = ld4f(yd + o + c); vd.x += t.x; vd.y += t.y; vd.z += t.z; vd.w += t.w; }
+      xds[k] = vd;
+    }
+  };
+  float s2 = 0.f, s1 = 0.f;
+  if constexpr (NC > 0) row_quads<NC>(d, lane, load);
+  row_quads<NC>(d, lane, [&](int k, int c) {
+    if constexpr (NC == 0) load(k, c);
+    const float4 v = xs[k];
+    *reinterpret_cast<float4*>(x_out + o + c) = v;
+    s2 += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+    if constexpr (DUAL) {
+      const float4 vd = xds[k];
       *reinterpret_cast<float4*>(xd_out + o + c) = vd;
       s1 += v.x * vd.x + v.y * vd.y + v.z * vd.z + v.w * vd.w;
     }
-  }
+  });
   s2 = warp_sum_all(s2);
   s1 = warp_sum_all(s1);
   const float inv_d = 1.f / static_cast<float>(d);
@@ -181,21 +207,21 @@ __global__ void __launch_bounds__(256) rmsnorm_fwd_warp_kernel(
   const float rsd = -rs * rs * rs * s1 * inv_d;
   if (lane == 0) {
     rr[r] = rs;
-    if (dual) rrd[r] = rsd;
+    if (DUAL) rrd[r] = rsd;
   }
   const int64_t oh = static_cast<int64_t>(r) * ldh;
-  for (int c = lane * 4; c < d; c += 128) {
-    const float4 v = ld4f(x_out + o + c), gg = ld4f(g + c);
+  row_quads<NC>(d, lane, [&](int k, int c) {
+    const float4 v = NC > 0 ? xs[k] : ld4f(x_out + o + c), gg = ld4f(g + c);
     const float n0 = v.x * rs, n1 = v.y * rs, n2 = v.z * rs, n3 = v.w * rs;
     st_t4<T>(h + oh + c, gg.x * n0, gg.y * n1, gg.z * n2, gg.w * n3);
-    if (dual) {
-      const float4 vd = ld4f(xd_out + o + c), ggd = ld4f(gd + c);
+    if constexpr (DUAL) {
+      const float4 vd = NC > 0 ? xds[k] : ld4f(xd_out + o + c), ggd = ld4f(gd + c);
       const float m0 = vd.x * rs + v.x * rsd, m1 = vd.y * rs + v.y * rsd;
       const float m2 = vd.z * rs + v.z * rsd, m3 = vd.w * rs + v.w * rsd;
       st_t4<T>(hd + oh + c, ggd.x * n0 + gg.x * m0, ggd.y * n1 + gg.y * m1,
                ggd.z * n2 + gg.z * m2, ggd.w * n3 + gg.w * m3);
     }
-  }
+  });
 }
 
 // Row r of the warp-per-row RMSNorm backward (this lane's columns lane*4 + 128 k).
@@ -317,6 +343,133 @@ __global__ void __launch_bounds__(256) rmsnorm_bwd_warp_kernel(
     const int64_t po = static_cast<int64_t>(blockIdx.x) * d + c;
     *reinterpret_cast<float4*>(part + po) = a;
     if (dual) *reinterpret_cast<float4*>(partd + po) = ad;
+  }
+}
+
+// Rows of up to 1024 VPT columns: a block walks its eight rows with one column group of four
+// per thread (VPT of them, 4 blockDim.x apart), so that the row's operands stay in registers
+// between the row sums and the result, the next row's loads are in flight meanwhile, and the
+// gain's partial sums accumulate in the order of the rows.  One barrier a row (the sums of the
+// warps in two alternating slots).  Memory bounds it: a dual call of 8192 x 1024 moves 310 MB
+// in 50 us (the warp kernel, which reads the operands again for the result and for the gain:
+// 69 us).
+template <typename T, bool DUAL, int VPT>
+__global__ void __launch_bounds__(256) rmsnorm_bwd_block_kernel(
+    int N, int d, const float* __restrict__ x, const float* __restrict__ xd,
+    const float* __restrict__ rr, const float* __restrict__ rrd, const float* __restrict__ g,
+    const float* __restrict__ gd, const float* __restrict__ dy, const float* __restrict__ dyd,
+    float* __restrict__ dx, float* __restrict__ dxd, T* __restrict__ dxb, T* __restrict__ dxdb,
+    float* __restrict__ part, float* __restrict__ partd, bool add) {
+  pdl_entry();
+  __shared__ float2 red[2][8];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int q0 = blockIdx.x * 8, q1 = min(N, q0 + 8);
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  struct Row { float4 x, dy, o, xd, dyd, od; float r, rd; };
+  Row nx[VPT];
+  float4 gg[VPT], ge[VPT], ga[VPT], gad[VPT];
+  auto col = [&](int k) { return 4 * static_cast<int>(threadIdx.x + k * blockDim.x); };
+  auto load = [&](int q) {
+#pragma unroll
+    for (int k = 0; k < VPT; ++k) {
+      const int c = col(k);
+      if (c >= d) continue;
+      const int64_t o = static_cast<int64_t>(q) * d + c;
+      nx[k].x = ld4f(x + o);
+      nx[k].dy = ld4f(dy + o);
+      if (add) nx[k].o = ld4f(dx + o);
+      if (DUAL) {
+        nx[k].xd = ld4f(xd + o);
+        nx[k].dyd = ld4f(dyd + o);
+        if (add) nx[k].od = ld4f(dxd + o);
+      }
+    }
+    nx[0].r = rr[q];
+    nx[0].rd = DUAL ? rrd[q] : 0.f;
+  };
+#pragma unroll
+  for (int k = 0; k < VPT; ++k) {
+    const bool on = col(k) < d;
+    nx[k].x = nx[k].dy = nx[k].o = nx[k].xd = nx[k].dyd = nx[k].od = zero;
+    gg[k] = on ? ld4f(g + col(k)) : zero;
+    ge[k] = DUAL && on ? ld4f(gd + col(k)) : zero;
+    ga[k] = gad[k] = zero;
+  }
+  load(q0);
+  const float inv_d = 1.f / static_cast<float>(d);
+  for (int q = q0; q < q1; ++q) {
+    Row v[VPT];
+#pragma unroll
+    for (int k = 0; k < VPT; ++k) v[k] = nx[k];
+    if (q + 1 < q1) load(q + 1);
+    const float rs = v[0].r, rsd = v[0].rd;
+    float n[VPT][4], nd[VPT][4], dn[VPT][4], dnd[VPT][4];
+    float sc = 0.f, scd = 0.f;
+#pragma unroll
+    for (int k = 0; k < VPT; ++k) {
+      const float xs[4] = {v[k].x.x, v[k].x.y, v[k].x.z, v[k].x.w};
+      const float ds[4] = {v[k].dy.x, v[k].dy.y, v[k].dy.z, v[k].dy.w};
+      const float xds[4] = {v[k].xd.x, v[k].xd.y, v[k].xd.z, v[k].xd.w};
+      const float dds[4] = {v[k].dyd.x, v[k].dyd.y, v[k].dyd.z, v[k].dyd.w};
+      const float gs[4] = {gg[k].x, gg[k].y, gg[k].z, gg[k].w};
+      const float gds[4] = {ge[k].x, ge[k].y, ge[k].z, ge[k].w};
+      float* a = &ga[k].x;
+      float* ad = &gad[k].x;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        n[k][j] = xs[j] * rs;
+        dn[k][j] = ds[j] * gs[j];
+        sc += dn[k][j] * n[k][j];
+        a[j] += ds[j] * n[k][j];
+        if (DUAL) {
+          nd[k][j] = xds[j] * rs + xs[j] * rsd;
+          dnd[k][j] = dds[j] * gs[j] + ds[j] * gds[j];
+          scd += dnd[k][j] * n[k][j] + dn[k][j] * nd[k][j];
+          ad[j] += dds[j] * n[k][j] + ds[j] * nd[k][j];
+        }
+      }
+    }
+    sc = warp_sum_all(sc);
+    if (DUAL) scd = warp_sum_all(scd);
+    if (lane == 0) red[q & 1][w] = make_float2(sc, scd);
+    __syncthreads();
+    float cc = 0.f, ccd = 0.f;
+    for (int i = 0; i < nw; ++i) {
+      const float2 t = red[q & 1][i];
+      cc += t.x;
+      ccd += t.y;
+    }
+    cc *= inv_d;
+    ccd *= inv_d;
+#pragma unroll
+    for (int k = 0; k < VPT; ++k) {
+      const int c = col(k);
+      if (c >= d) continue;
+      const int64_t o = static_cast<int64_t>(q) * d + c;
+      const float os[4] = {v[k].o.x, v[k].o.y, v[k].o.z, v[k].o.w};
+      const float ods[4] = {v[k].od.x, v[k].od.y, v[k].od.z, v[k].od.w};
+      float out[4], outd[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float t = dn[k][j] - n[k][j] * cc;
+        out[j] = os[j] + rs * t;
+        if (DUAL) outd[j] = ods[j] + rsd * t + rs * (dnd[k][j] - nd[k][j] * cc - n[k][j] * ccd);
+      }
+      *reinterpret_cast<float4*>(dx + o) = make_float4(out[0], out[1], out[2], out[3]);
+      if (dxb) st_t4<T>(dxb + o, out[0], out[1], out[2], out[3]);
+      if constexpr (DUAL) {
+        *reinterpret_cast<float4*>(dxd + o) = make_float4(outd[0], outd[1], outd[2], outd[3]);
+        if (dxdb) st_t4<T>(dxdb + o, outd[0], outd[1], outd[2], outd[3]);
+      }
+    }
+  }
+  if (!part) return;
+#pragma unroll
+  for (int k = 0; k < VPT; ++k) {
+    if (col(k) >= d) continue;
+    const int64_t po = static_cast<int64_t>(blockIdx.x) * d + col(k);
+    *reinterpret_cast<float4*>(part + po) = ga[k];
+    if (DUAL) *reinterpret_cast<float4*>(partd + po) = gad[k];
   }
 }
 
@@ -477,13 +630,13 @@ __device__ __forceinline__ void store4<__nv_bfloat16>(__nv_bfloat16* p, float a,
 // v, their partners and two (cos, sin) pairs of the table; 8-byte (bf16) stores.
 template <typename T>
 __global__ void rope_split_kernel(int S, int H, int dh, const float* __restrict__ rtab, float qscale,
-                                  const float* __restrict__ qkv, T* __restrict__ Q,
-                                  T* __restrict__ K, T* __restrict__ Vv) {
+                                  RopeSplit<T> a, RopeSplit<T> b2) {
   pdl_entry();
   const int r = blockIdx.x;                 // token row
+  const RopeSplit<T> t = blockIdx.y ? b2 : a;
   const int b = r / S, s = r % S;
   const int d = H * dh, half = dh / 2;
-  const float* row = qkv + static_cast<int64_t>(r) * 3 * d;
+  const float* row = t.qkv + static_cast<int64_t>(r) * 3 * d;
   for (int c = 4 * threadIdx.x; c < d; c += 4 * blockDim.x) {
     const int h = c / dh, e = c % dh;
     const bool lo = e < half;
@@ -507,9 +660,9 @@ __global__ void rope_split_kernel(int S, int H, int dh, const float* __restrict_
       ko[i] = ka[i] * cs[i] + sg * kb[i] * sn[i];
     }
     const int64_t o = ((static_cast<int64_t>(b) * H + h) * S + s) * dh + e;
-    store4<T>(Q + o, qo[0], qo[1], qo[2], qo[3]);
-    store4<T>(K + o, ko[0], ko[1], ko[2], ko[3]);
-    store4<T>(Vv + o, v.x, v.y, v.z, v.w);
+    store4<T>(t.Q + o, qo[0], qo[1], qo[2], qo[3]);
+    store4<T>(t.K + o, ko[0], ko[1], ko[2], ko[3]);
+    store4<T>(t.V + o, v.x, v.y, v.z, v.w);
   }
 }
 
@@ -1096,8 +1249,23 @@ void dec_rmsnorm_fwd(int N, int d, float eps, const float* x_in, const float* y,
                   reinterpret_cast<uintptr_t>(x_out) | reinterpret_cast<uintptr_t>(xd_out) |
                   reinterpret_cast<uintptr_t>(h) | reinterpret_cast<uintptr_t>(hd);
   if ((any & 15) == 0 && (d & 3) == 0 && (ldh & 7) == 0) {
-    launch_k(rmsnorm_fwd_warp_kernel<T>, dim3((N + 7) / 8), dim3(256), 0, s, N, d, eps, x_in, y,
-             xd_in, yd, g, gd, x_out, xd_out, r, rd, h, hd, ldh);
+    auto go = [&](auto dual, auto nc) {
+      launch_k(rmsnorm_fwd_warp_kernel<T, decltype(dual)::value, decltype(nc)::value>,
+               dim3((N + 7) / 8), dim3(256), 0, s, N, d, eps, x_in, y, xd_in, yd, g, gd, x_out,
+               xd_out, r, rd, h, hd, ldh);
+    };
+    auto width = [&](auto dual) {
+      if (d <= 256) go(dual, std::integral_constant<int, 2>{});
+      else if (d <= 512) go(dual, std::integral_constant<int, 4>{});
+      else if (d <= 768) go(dual, std::integral_constant<int, 6>{});
+      else if (d <= 1024) go(dual, std::integral_constant<int, 8>{});
+      else go(dual, std::integral_constant<int, 0>{});
+    };
+    // rows in registers wherever they fit: 4096 x 512 11.10 -> 11.04 ms a call for the dual
+    // forward and -> 11.00 for the primal one, a 1200 x 768 Hessian-vector product 1608 ->
+    // 1584 us, a 2048 x 1024 one 2685 -> 2640 us
+    if (xd_in) width(std::true_type{});
+    else width(std::false_type{});
     return;
   }
   launch_k(rmsnorm_fwd_kernel<T>, dim3(N), dim3(256), 0, s, d, eps, x_in, y, xd_in, yd, g, gd, x_out, xd_out, r, rd,
@@ -1122,8 +1290,31 @@ int dec_rmsnorm_bwd(int N, int d, const float* x, const float* xd, const float* 
     const int nblk = (N + 7) / 8;
     float* pp = gain ? part : nullptr;
     float* ppd = gain && dyd ? part + static_cast<int64_t>(nblk) * d : nullptr;
-    launch_k(rmsnorm_bwd_warp_kernel<T>, dim3(nblk), dim3(256), 0, s, N, d, x, xd, r, rd, g, gd,
-             dy, dyd, dx, dxd, dxb, dxdb, pp, ppd, add);
+    auto block = [&](auto dual, auto vpt) {
+      constexpr int V = decltype(vpt)::value;
+      const int threads = (d + 128 * V - 1) / (128 * V) * 32;
+      launch_k(rmsnorm_bwd_block_kernel<T, decltype(dual)::value, V>, dim3(nblk), dim3(threads), 0,
+               s, N, d, x, xd, r, rd, g, gd, dy, dyd, dx, dxd, dxb, dxdb, pp, ppd, add);
+    };
+    auto width = [&](auto dual) {
+      if (d <= 1024) block(dual, std::integral_constant<int, 1>{});
+      else block(dual, std::integral_constant<int, 2>{});
+    };
+    // Rows of 257 to 2048 columns go to the block kernel; against the warp kernel, which reads
+    // a row's operands three times, a 4096-token 512-wide decoder's whole call took 11.10 ->
+    // 10.97 ms with the block kernel for its dual backward and 11.10 with it for the primal
+    // one, 8192 x 1024 166.0 -> 164.6 and -> 164.8 ms, a 1200 x 768 Hessian-vector product
+    // 1608 -> 1591 us.  Shorter rows leave the block kernel's threads idle (256 x 64: 2.6
+    // against 4.7 us a launch).
+    const bool by_warps = d <= 256 || d > 2048;
+    if (by_warps) {
+      launch_k(rmsnorm_bwd_warp_kernel<T>, dim3(nblk), dim3(256), 0, s, N, d, x, xd, r, rd, g, gd,
+               dy, dyd, dx, dxd, dxb, dxdb, pp, ppd, add);
+    } else if (dyd) {
+      width(std::true_type{});
+    } else {
+      width(std::false_type{});
+    }
     return nblk;
   }
   launch_k(rmsnorm_bwd_kernel<T>, dim3(N), dim3(256), 0, s, d, x, xd, r, rd, g, gd, dy, dyd, dx, dxd,
@@ -1151,9 +1342,12 @@ void dec_rope_table(int S, int dh, float base, float* tab, cudaStream_t s) {
 }
 
 template <typename T>
-void dec_rope_split(int N, int S, int H, int dh, const float* rtab, float qscale, const float* qkv,
-                    T* Q, T* K, T* V, cudaStream_t s) {
-  launch_k(rope_split_kernel<T>, dim3(N), dim3(256), 0, s, S, H, dh, rtab, qscale, qkv, Q, K, V);
+void dec_rope_split(int N, int S, int H, int dh, const float* rtab, float qscale,
+                    const RopeSplit<T>& a, const RopeSplit<T>& b, cudaStream_t s) {
+  // one thread per four columns (a block of 256 left half its threads idle at d = 512)
+  const int threads = H * dh >= 1024 ? 256 : (H * dh / 4 + 31) / 32 * 32;
+  launch_k(rope_split_kernel<T>, dim3(N, b.qkv ? 2 : 1), dim3(threads), 0, s, S, H, dh, rtab,
+           qscale, a, b);
 }
 
 template <typename T>
@@ -1239,8 +1433,8 @@ void cast_rows(const float* X, int rows, int cols, T* Y, int ldy, cudaStream_t s
                                   const float*, const float*, const float*, const float*,          \
                                   const float*, float*, float*, bool, bool, float*, cudaStream_t,  \
                                   T*, T*);                                           \
-  template void dec_rope_split<T>(int, int, int, int, const float*, float, const float*, T*, T*, T*,      \
-                                  cudaStream_t);                                                   \
+  template void dec_rope_split<T>(int, int, int, int, const float*, float, const RopeSplit<T>&,    \
+                                  const RopeSplit<T>&, cudaStream_t);                              \
   template void dec_rope_merge<T>(int, int, int, int, const float*, float, const float*, const float*,    \
                                   const float*, T*, int, cudaStream_t);                            \
   template void dec_head_merge<T>(int, int, int, int, const float*, T*, int, cudaStream_t);       \

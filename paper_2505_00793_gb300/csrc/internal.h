@@ -379,9 +379,15 @@ void dec_gain_final(int nchunk, int d, bool dual, const float* part, float* dg, 
                     cudaStream_t s);
 // RoPE table [S][dh/2] of (cos, sin) pairs, float32, from double-precision angles.
 void dec_rope_table(int S, int dh, float base, float* tab, cudaStream_t s);
+// Two projections in one launch (the second with qkv set: the tangent's).
 template <typename T>
-void dec_rope_split(int N, int S, int H, int dh, const float* rtab, float qscale, const float* qkv,
-                    T* Q, T* K, T* V, cudaStream_t s);
+struct RopeSplit {
+  const float* qkv = nullptr;
+  T *Q = nullptr, *K = nullptr, *V = nullptr;
+};
+template <typename T>
+void dec_rope_split(int N, int S, int H, int dh, const float* rtab, float qscale,
+                    const RopeSplit<T>& a, const RopeSplit<T>& b, cudaStream_t s);
 template <typename T>
 void dec_rope_merge(int N, int S, int H, int dh, const float* rtab, float qscale, const float* dQ,
                     const float* dK, const float* dV, T* out, int ldo, cudaStream_t s);

@@ -43,3 +43,32 @@ def test_decoder_backward_passes(V, shift, side):
         assert rel_l2(g.cpu().numpy(), om.grad(w, inp.theta0, ids, ids, wt)) < 1e-4
         assert rel_l2(Hv.cpu().numpy(), om.hvp(w, inp.theta0, ids, ids, v, wt)) < 1e-4
     mf.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d,H,rows,S", [(264, 33, 1, 16), (520, 65, 5, 24), (776, 97, 3, 200),
+                                        (1024, 16, 2, 616), (1032, 129, 2, 16),
+                                        (1024, 16, 8, 520), (2056, 257, 1, 8)])
+def test_norm_widths(d, H, rows, S):
+    """RMSNorm kernels by row width and batch: rows kept by a warp, by a block (one and two
+    column groups a thread, ragged ends, fewer than eight rows in the last block), and walked;
+    primal and dual (both schedules), on either side of the rules that choose."""
+    torch, native = need_gpu()
+    from oracle import metagrad as om
+    w = synth.decoder("norms", d, H, 8, 1, 16, S, B=rows, T=1, B_outer=1,
+                      alpha=0.1).with_(precision="fp32")
+    inp = synth.make_inputs(w)
+    ids = inp.inner_x[0]
+    v = synth.random_direction(w.n_params, 2, 3)
+    one = np.ones(w.B, np.float32)
+    d_in = native.to_device_inputs(w, inp)
+    mf = native.MixFlow.for_workload(w)
+    ref = om.grad(w, inp.theta0, ids, ids, one), om.hvp(w, inp.theta0, ids, ids, v, one)
+    for mode in (native.MF_HVP_MIXED_FOR, native.MF_HVP_REV_REV):
+        Hv, g = (torch.full((w.n_params,), float("nan"), device="cuda") for _ in range(2))
+        mf.hvp(w.B, d_in["theta0"], d_in["inner_x"][0], d_in["inner_y"][0],
+               torch.from_numpy(v).cuda(), Hv, grad=g, hvp_mode=mode)
+        mf.sync()
+        assert rel_l2(g.cpu().numpy(), ref[0]) < 1e-4
+        assert rel_l2(Hv.cpu().numpy(), ref[1]) < 1e-4
+    mf.close()
