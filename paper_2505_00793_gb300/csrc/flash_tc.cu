@@ -111,10 +111,6 @@ __device__ __forceinline__ void tmem_ld32_nowait(uint32_t taddr, float* v) {
 #pragma unroll
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
-__device__ __forceinline__ void tmem_wait_ld() {
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
 // Pairs of float32: sm_103a runs an operation on both halves as one instruction, each rounded
 // as the scalar operation is.
 __device__ __forceinline__ uint64_t pair(float a, float b) {
@@ -637,20 +633,6 @@ struct FtbParams {
   const float* rope;
   float qscale;
 };
-
-// One 16-column TMEM load without its wait, so that several are in flight.
-__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, float (&v)[16]) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-        "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
 
 // Columns cb .. cb + CW - 1 of a 128 x 64 float32 accumulator row (this thread's TMEM lane) to
 // global memory.

@@ -245,6 +245,24 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// One 16-column TMEM load without its wait, so that several are in flight.
+__device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, float (&v)[16]) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
+        "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+__device__ __forceinline__ void tmem_wait_ld() {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
 // Accumulators.  Logical accumulator c (0: C0, 1: C1) owns nsub blocks of BN TMEM columns
 // at (c * nsub + j) * BN.  Successive products into one logical accumulator rotate over its
 // blocks: an MMA into a block waits for the previous MMA into the same block (its
@@ -259,6 +277,29 @@ __device__ __forceinline__ void ld_acc16(uint32_t taddr, int c, int nsub, int co
     tmem_ld16(taddr + static_cast<uint32_t>((c * nsub + j) * BN + col), t);
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] += t[i];
+  }
+}
+// Keeps the uses of values loaded without a wait behind the wait.
+__device__ __forceinline__ void loaded16(float (&v)[16]) {
+  asm volatile("" : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]),
+               "+f"(v[6]), "+f"(v[7]), "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]),
+               "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15]));
+}
+// The same with the loads of all blocks in flight together.
+template <int BN, int NSUB>
+__device__ __forceinline__ void ld_acc16_all(uint32_t taddr, int c, int col, float (&v)[16]) {
+  float t[NSUB][16];
+#pragma unroll
+  for (int j = 0; j < NSUB; ++j)
+    tmem_ld16_nowait(taddr + static_cast<uint32_t>((c * NSUB + j) * BN + col), t[j]);
+  tmem_wait_ld();
+#pragma unroll
+  for (int j = 0; j < NSUB; ++j) loaded16(t[j]);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    v[i] = t[0][i];
+#pragma unroll
+    for (int j = 1; j < NSUB; ++j) v[i] += t[j][i];
   }
 }
 
@@ -945,9 +986,16 @@ __device__ __forceinline__ void mma_dispatch(const MmaLoop& L, unsigned terms, i
 // complete a barrier there, the sum is fused with the epilogue at four columns of one row per
 // thread, and the stored inputs load during the main loop.  Wide MLP meta-gradient (462 such
 // GEMMs) 5.33 -> 4.31 ms, ragged reverse-over-reverse step 240 -> 202 us, transformer with
-// 96-wide heads 1.96 -> 1.75 ms.
+// 96-wide heads 1.96 -> 1.75 ms.  Of the 15,000 clocks of a 256 x 1024 x 1024 dual product split
+// four ways, the main loop takes 5,400 (L2 reads) and the exchange 2,700; the accumulator
+// blocks are loaded together, the partial sums of a quad too, and only warps with something
+// to publish release the cluster barriers (9.25 -> 8.5 us in a chain of such products, with
+// stored derivatives 8.6 -> 7.8; the wide meta-gradient 4.22 -> 3.95 ms).
 __device__ __forceinline__ void cluster_arrive() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_arrive_relaxed() {
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -1176,7 +1224,10 @@ __global__ void __launch_bounds__(THREADS, 1)
     const bool ok = nk > 0 && mbar_wait(&acc_bar, 0, p.status, p.wait_ns);
     // a peer waits for this CTA's partial sums whether or not the wait gave up
     if (S > 1 && nk > 0 && !ok) mbar_wait(&acc_bar, 0, p.status, DRAIN_NS);
-    if (S > 1) cluster_arrive();
+    // the pipeline buffers are free: warps 0 and 1, which saw the last loads and products
+    // complete, release that; these warps have nothing to publish (a releasing arrive took
+    // 1,000 clocks)
+    if (S > 1) cluster_arrive_relaxed();
     tc_fence_after();
     auto fill = [&](int cb) {   // columns [cb, cb + CW) of the accumulators into the tile
       for (int a = 0; a < nacc; ++a)
@@ -1184,7 +1235,10 @@ __global__ void __launch_bounds__(THREADS, 1)
         for (int c = ((warp - 2) >> 2) * 16; c < CW; c += 16 * EPI_GROUPS) {
           float v[16];
           if (nk > 0) {
-            ld_acc16<BN>(tbase + lane_off, a, p.nsub, cb + c, v);
+            const uint32_t t = tbase + lane_off;
+            if (p.nsub == 4) ld_acc16_all<BN, 4>(t, a, cb + c, v);
+            else if (p.nsub == 2) ld_acc16_all<BN, 2>(t, a, cb + c, v);
+            else ld_acc16_all<BN, 1>(t, a, cb + c, v);
           } else {
 #pragma unroll
             for (int q = 0; q < 16; ++q) v[q] = 0.f;
@@ -1237,31 +1291,40 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
       __syncwarp();
       mbar_wait(&recv_bar, 0, p.status, DRAIN_NS);
-      cluster_arrive();   // the peers' copies out of their tiles to this CTA are complete
+      // the peers' copies out of their tiles to this CTA are complete (nothing is published:
+      // a releasing arrive took 1,000 clocks)
+      cluster_arrive_relaxed();
+      // the S partial sums of a quad, read together and added in rank order
+      auto finish = [&](auto split) {
+        constexpr int NS = decltype(split)::value;
 #pragma unroll 1
-      for (int u = e; u < rows_per * VPR; u += EPI_THREADS) {
-        const int row = u / VPR, col = u % VPR * 4;
-        const int m = m0 + r_begin + row, n = n0 + col;
-        if (u != e) epi_load<MODE>(in0, p, m, n, dual);
-        float4 x[2];
-        x[1] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int u = e; u < rows_per * VPR; u += EPI_THREADS) {
+          const int row = u / VPR, col = u % VPR * 4;
+          const int m = m0 + r_begin + row, n = n0 + col;
+          if (u != e) epi_load<MODE>(in0, p, m, n, dual);
+          float4 x[2];
+          x[1] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int a = 0; a < 2; ++a) {
-          if (a == nacc) break;
-          const float4 own = *reinterpret_cast<const float4*>(tile + ET::at(a * BM + r_begin + row, col));
-          float4 t = own;
-          for (int k = 0; k < S; ++k) {
-            float4 v = own;
-            if (k != zs)
-              v = *reinterpret_cast<const float4*>(
-                  recv + ET::at((a * (S - 1) + (k < zs ? k : k - 1)) * rows_per + row, col));
-            if (k == 0) t = v;
-            else { t.x += v.x; t.y += v.y; t.z += v.z; t.w += v.w; }
+          for (int a = 0; a < 2; ++a) {
+            if (a == nacc) break;
+            float4 v[NS];
+#pragma unroll
+            for (int k = 0; k < NS; ++k)
+              v[k] = *reinterpret_cast<const float4*>(
+                  k == zs ? tile + ET::at(a * BM + r_begin + row, col)
+                          : recv + ET::at((a * (NS - 1) + (k < zs ? k : k - 1)) * rows_per + row, col));
+            x[a] = v[0];
+#pragma unroll
+            for (int k = 1; k < NS; ++k) {
+              x[a].x += v[k].x; x[a].y += v[k].y; x[a].z += v[k].z; x[a].w += v[k].w;
+            }
           }
-          x[a] = t;
+          epi_quad<MODE, ACT>(p, m, n, x[0], x[1], in0, dual);
         }
-        epi_quad<MODE, ACT>(p, m, n, x[0], x[1], in0, dual);
-      }
+      };
+      if (S == 2) finish(std::integral_constant<int, 2>{});
+      else if (S == 4) finish(std::integral_constant<int, 4>{});
+      else finish(std::integral_constant<int, 8>{});
       __syncwarp();
       cluster_wait();
     }
