@@ -199,7 +199,12 @@ struct DecExec {
   }
 
   template <typename U> U* at(size_t off) const { return reinterpret_cast<U*>(base + off); }
-  float* theta_slot(int t) const { return at<float>(p.o_theta) + static_cast<int64_t>(t) * h->P; }
+  const float* theta0_ext = nullptr;   // theta_0, where the caller's vector serves as slot 0
+  bool in_place() const { return true; }
+  float* theta_slot(int t) const {
+    if (t == 0 && theta0_ext) return const_cast<float*>(theta0_ext);   // never written
+    return at<float>(p.o_theta) + static_cast<int64_t>(t) * h->P;
+  }
   float* m_slot(int j) const { return at<float>(p.o_m) + static_cast<int64_t>(j) * h->P; }
   float* g_buf() const { return at<float>(p.o_g); }
   float* tbar_buf() const { return at<float>(p.o_tbar); }

@@ -223,6 +223,7 @@ struct LayerUpdArgs {
   // LU_ADJOINT (K5):  theta_bar += Hu ; d eta_lr from m_adj ; u' = mu u - lr theta_bar ;
   //                   cast u' into U
   float* theta_bar = nullptr; const float* Hu = nullptr; const float* m_adj = nullptr;
+  float* theta_bar_out = nullptr;  // where theta_bar + Hu goes (null: theta_bar)
   const float* u_in = nullptr; float* u_out = nullptr; float* d_plr = nullptr;
   float* partials = nullptr;       // scalar log-lr: one partial per block (tile)
   bool plr_first = false;          // d_plr is written, not added to

@@ -592,7 +592,7 @@ __device__ __forceinline__ void layer_update_block(const LayerTable& tab, const 
         tb[j] += hu[j];
         bad |= j < cnt && !isfinite(tb[j]);
       }
-      st4(a.theta_bar, k, tb, vec, cnt);
+      st4(a.theta_bar_out ? a.theta_bar_out : a.theta_bar, k, tb, vec, cnt);
       float contrib[4] = {0.f, 0.f, 0.f, 0.f};
       bool have_contrib = false;
       if (a.adam && a.adam_pre) {
@@ -965,7 +965,8 @@ bool update_vec_ok(const LayerUpdArgs& a) {
   for (const void* p : {static_cast<const void*>(a.cast_src), static_cast<const void*>(a.theta),
                         static_cast<const void*>(a.m), static_cast<const void*>(a.g),
                         static_cast<const void*>(a.theta_out), static_cast<const void*>(a.m_out),
-                        static_cast<const void*>(a.theta_bar), static_cast<const void*>(a.Hu),
+                        static_cast<const void*>(a.theta_bar), static_cast<const void*>(a.theta_bar_out),
+                        static_cast<const void*>(a.Hu),
                         static_cast<const void*>(a.m_adj), static_cast<const void*>(a.u_in),
                         static_cast<const void*>(a.u_out), static_cast<const void*>(a.d_plr),
                         static_cast<const void*>(a.lr.plr), static_cast<const void*>(a.v),
