@@ -507,10 +507,27 @@ __device__ __forceinline__ void st_copy(T* W, int64_t e0, int r0, int dout, int 
 // serves the products, and the sum of the first learning-rate gradients.  Eight 4096-wide
 // layers, momentum, per-parameter rates, 32 steps: 8.08 -> 8.03 ms a call; 256-512-512-128,
 // 64 steps: 978 -> 957 us.
-template <typename T, class Sync>
+// One kernel per mode, so that each has the registers of its own vectors only, and its layer
+// table read from constant memory (a per-thread copy of it in local memory cost more than the
+// search for the layer): the same calls 7.33 -> 6.77 ms and 912 -> 846 us, a 1024-wide one
+// 3.92 -> 3.80 ms.
+#pragma nv_exec_check_disable
+template <class F>
+__host__ __device__ __forceinline__ void with_update_mode(const LayerUpdArgs& a, F&& f) {
+  using R = std::integral_constant<int, LU_ROLLOUT>;
+  using A = std::integral_constant<int, LU_ADJOINT>;
+  if (a.mode == LU_ROLLOUT && a.adam) f(R{}, std::true_type{});
+  else if (a.mode == LU_ROLLOUT) f(R{}, std::false_type{});
+  else if (a.mode == LU_ADJOINT && a.adam) f(A{}, std::true_type{});
+  else if (a.mode == LU_ADJOINT) f(A{}, std::false_type{});
+  else f(std::integral_constant<int, LU_CAST>{}, std::false_type{});
+}
+
+// Tiles blk .. blk + NQ - 1, whose loads are all issued before the first result is needed.
+template <typename T, int MODE, bool ADAM, int NQ, class Sync>
 __device__ __forceinline__ void layer_update_block(const LayerTable& tab, const LayerUpdArgs& a,
                                                    int blk, int tid, float* red, Sync sync) {
-  // the layer of this block: the last l with tile0[l] <= blk (binary search)
+  // the layer of the first tile: the last l with tile0[l] <= blk (binary search)
   int l = 0;
   {
     int hi = tab.n - 1;
@@ -520,18 +537,70 @@ __device__ __forceinline__ void layer_update_block(const LayerTable& tab, const 
       else hi = mid - 1;
     }
   }
-  const int dout = tab.dout[l], din = tab.din[l];
-  const int64_t n = static_cast<int64_t>(tab.rows[l]) * dout;
-  const int64_t e0 = (static_cast<int64_t>(blk - tab.tile0[l]) * UPD_THREADS + tid) * 4;
-  const bool cast_w = (a.mode == LU_ROLLOUT) || (a.mode == LU_CAST && !a.cast_src_to_u) ||
-                      (a.mode == LU_ADJOINT && a.cast_src);
-  const bool cast_u = (a.mode == LU_CAST && a.cast_src_to_u) || (a.mode == LU_ADJOINT && a.u_out);
+  struct Pos { int l, dout, cnt; bool vec; int64_t n, e0, k; };
+  auto place = [&](int lay, int q) {
+    Pos z;
+    z.l = lay;
+    z.dout = tab.dout[lay];
+    z.n = static_cast<int64_t>(tab.rows[lay]) * z.dout;
+    z.e0 = (static_cast<int64_t>(blk + q - tab.tile0[lay]) * UPD_THREADS + tid) * 4;
+    z.cnt = static_cast<int>(z.n - z.e0 < 4 ? z.n - z.e0 : 4);
+    z.vec = a.vec_ok && z.cnt == 4 && (tab.off[lay] & 3) == 0 && (z.dout & 3) == 0;
+    z.k = tab.off[lay] + z.e0;
+    return z;
+  };
+  const bool cast_w = (MODE == LU_ROLLOUT) || (MODE == LU_CAST && !a.cast_src_to_u) ||
+                      (MODE == LU_ADJOINT && a.cast_src);
+  const bool cast_u = (MODE == LU_CAST && a.cast_src_to_u) || (MODE == LU_ADJOINT && a.u_out);
+  const bool need_lr = MODE == LU_ROLLOUT ||
+                       (MODE == LU_ADJOINT && ((ADAM && a.adam_pre) || a.m_adj || a.u_out));
+  constexpr bool plain = !ADAM;
+  // Inputs of one tile: the rollout's theta, g, m, v; the adjoint's theta_bar, Hu and (plain)
+  // m_adj, u_in, d_plr, cast_src; the cast's source.  The pointers may alias in place, so
+  // every one of them is read before the tile's first store.
+  struct In { float lr[4], x0[4], x1[4], x2[4], x3[4], x4[4], x5[4]; } in[NQ];
+  int lay[NQ];
+  bool on[NQ];
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    if (q > 0)
+      while (l + 1 < tab.n && blk + q >= tab.tile0[l + 1]) ++l;
+    lay[q] = l;
+    const Pos z = place(l, q);
+    on[q] = z.e0 < z.n;
+    In& i = in[q];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      i.lr[j] = i.x0[j] = i.x1[j] = i.x2[j] = i.x3[j] = i.x4[j] = i.x5[j] = 0.f;
+    if (!on[q]) continue;
+    if (a.lr.plr && need_lr) ld4(i.lr, a.lr.plr, z.k, z.vec, z.cnt);
+    if (MODE == LU_ROLLOUT) {
+      ld4(i.x0, a.theta, z.k, z.vec, z.cnt);
+      ld4(i.x1, a.g, z.k, z.vec, z.cnt);
+      if (a.m) ld4(i.x2, a.m, z.k, z.vec, z.cnt);
+      if (ADAM && a.v) ld4(i.x3, a.v, z.k, z.vec, z.cnt);
+    } else if (MODE == LU_ADJOINT) {
+      ld4(i.x0, a.theta_bar, z.k, z.vec, z.cnt);
+      if (a.Hu) ld4(i.x1, a.Hu, z.k, z.vec, z.cnt);
+      if (plain && a.m_adj) ld4(i.x2, a.m_adj, z.k, z.vec, z.cnt);
+      if (plain && a.u_out && a.u_in) ld4(i.x3, a.u_in, z.k, z.vec, z.cnt);
+      if (plain && a.m_adj && a.d_plr && !a.plr_first) ld4(i.x4, a.d_plr, z.k, z.vec, z.cnt);
+      if (plain && a.cast_src) ld4(i.x5, a.cast_src, z.k, z.vec, z.cnt);
+    } else {
+      ld4(i.x0, a.cast_src, z.k, z.vec, z.cnt);
+    }
+  }
   bool bad = false;
-  float acc = 0.f;
-  if (e0 < n) {
-    const int cnt = static_cast<int>(n - e0 < 4 ? n - e0 : 4);
-    const bool vec = a.vec_ok && cnt == 4 && (tab.off[l] & 3) == 0 && (dout & 3) == 0;
-    const int64_t k = tab.off[l] + e0;
+  float acc[NQ];
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    acc[q] = 0.f;
+    if (!on[q]) continue;
+    const Pos z = place(lay[q], q);
+    const int l = z.l, dout = z.dout, cnt = z.cnt, din = tab.din[l];
+    const bool vec = z.vec;
+    const int64_t n = z.n, e0 = z.e0, k = z.k;
+    In& i = in[q];
     // the float32 tangent of an element that its operand copy serves (the quads of a vector
     // access lie in one row)
     const int r0 = n <= 0xffffffffLL
@@ -540,27 +609,20 @@ __device__ __forceinline__ void layer_update_block(const LayerTable& tab, const 
     const bool u_kept = !(a.u_copy && vec && tab.U[l] && r0 < din);
     float vw[4] = {0.f, 0.f, 0.f, 0.f}, vu[4] = {0.f, 0.f, 0.f, 0.f};
     float lr[4];
-    const bool need_lr = a.mode == LU_ROLLOUT ||
-                         (a.mode == LU_ADJOINT && (a.adam_pre || a.m_adj || a.u_out));
     if (a.lr.plr && need_lr) {
-      ld4(lr, a.lr.plr, k, vec, cnt);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) lr[j] = expf(lr[j]);
+      for (int j = 0; j < 4; ++j) lr[j] = expf(i.lr[j]);
     } else {
       const float l0 = a.lr.slr ? expf(a.lr.slr[0]) : a.lr.alpha;
 #pragma unroll
       for (int j = 0; j < 4; ++j) lr[j] = l0;
     }
-    if (a.mode == LU_ROLLOUT) {
-      float th[4], g[4], m[4] = {0.f, 0.f, 0.f, 0.f}, v[4] = {0.f, 0.f, 0.f, 0.f};
-      ld4(th, a.theta, k, vec, cnt);
-      ld4(g, a.g, k, vec, cnt);
-      if (a.m) ld4(m, a.m, k, vec, cnt);
-      if (a.adam && a.v) ld4(v, a.v, k, vec, cnt);
+    if (MODE == LU_ROLLOUT) {
+      const float(&th)[4] = i.x0, (&g)[4] = i.x1, (&m)[4] = i.x2, (&v)[4] = i.x3;
       float mn[4], vn[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        if (a.adam) {
+        if (ADAM) {
           mn[j] = a.b1 * m[j] + (1.f - a.b1) * g[j];
           vn[j] = a.b2 * v[j] + (1.f - a.b2) * g[j] * g[j];
           vw[j] = th[j] - lr[j] * (mn[j] / a.c1) / (sqrtf(vn[j] / a.c2) + a.eps);
@@ -573,20 +635,14 @@ __device__ __forceinline__ void layer_update_block(const LayerTable& tab, const 
       }
       st4(a.theta_out, k, vw, vec, cnt);
       if (a.m_out) st4(a.m_out, k, mn, vec, cnt);
-      if (a.adam && a.v_out) st4(a.v_out, k, vn, vec, cnt);
-    } else if (a.mode == LU_ADJOINT) {
-      float tb[4], hu[4] = {0.f, 0.f, 0.f, 0.f};
-      ld4(tb, a.theta_bar, k, vec, cnt);
-      if (a.Hu) ld4(hu, a.Hu, k, vec, cnt);
-      // every other input of the plain (non-Adam) adjoint is loaded before the first store,
-      // so that a thread's loads are in flight together (the pointers may alias in place)
-      float ma[4] = {0.f, 0.f, 0.f, 0.f}, ui[4] = {0.f, 0.f, 0.f, 0.f};
-      float dp[4] = {0.f, 0.f, 0.f, 0.f};
-      const bool plain = !a.adam;
-      if (plain && a.m_adj) ld4(ma, a.m_adj, k, vec, cnt);
-      if (plain && a.u_out && a.u_in) ld4(ui, a.u_in, k, vec, cnt);
-      if (plain && a.m_adj && a.d_plr && !a.plr_first) ld4(dp, a.d_plr, k, vec, cnt);
-      if (plain && a.cast_src) ld4(vw, a.cast_src, k, vec, cnt);
+      if (ADAM && a.v_out) st4(a.v_out, k, vn, vec, cnt);
+    } else if (MODE == LU_ADJOINT) {
+      float(&tb)[4] = i.x0, (&dp)[4] = i.x4;
+      const float(&hu)[4] = i.x1, (&ma)[4] = i.x2, (&ui)[4] = i.x3;
+      if (plain && a.cast_src) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) vw[j] = i.x5[j];
+      }
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         tb[j] += hu[j];
@@ -595,7 +651,7 @@ __device__ __forceinline__ void layer_update_block(const LayerTable& tab, const 
       st4(a.theta_bar_out ? a.theta_bar_out : a.theta_bar, k, tb, vec, cnt);
       float contrib[4] = {0.f, 0.f, 0.f, 0.f};
       bool have_contrib = false;
-      if (a.adam && a.adam_pre) {
+      if (ADAM && a.adam_pre) {
         // reverse of Adam step j from its outputs m1 = m_{j+1}, v1 = v_{j+1} (see LayerUpdArgs)
         float m1[4], v1[4], mp[4] = {0.f, 0.f, 0.f, 0.f};
         float mb[4] = {0.f, 0.f, 0.f, 0.f}, vb[4] = {0.f, 0.f, 0.f, 0.f};
@@ -610,10 +666,10 @@ __device__ __forceinline__ void layer_update_block(const LayerTable& tab, const 
         for (int j = 0; j < 4; ++j) {
           const float sq = sqrtf(v1[j] / a.c2);
           const float den = sq + a.eps;
-          const float q = -lr[j] * tb[j];
+          const float s = -lr[j] * tb[j];
           // at v = 0 (where m = g = 0) the sqrt term is 0
-          const float Mb = mb[j] + q / (a.c1 * den);
-          const float Vb = vb[j] - (sq > 0.f ? q * m1[j] / (a.c1 * den * den * 2.f * sq * a.c2) : 0.f);
+          const float Mb = mb[j] + s / (a.c1 * den);
+          const float Vb = vb[j] - (sq > 0.f ? s * m1[j] / (a.c1 * den * den * 2.f * sq * a.c2) : 0.f);
           const float g = (m1[j] - a.b1 * mp[j]) / (1.f - a.b1);
           vu[j] = (1.f - a.b1) * Mb + 2.f * (1.f - a.b2) * g * Vb;
           mb[j] = a.b1 * Mb;
@@ -645,39 +701,44 @@ __device__ __forceinline__ void layer_update_block(const LayerTable& tab, const 
           st4(a.d_plr, k, dp, vec, cnt);
         } else {
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc += j < cnt ? contrib[j] : 0.f;
+          for (int j = 0; j < 4; ++j) acc[q] += j < cnt ? contrib[j] : 0.f;
         }
       }
       if (!plain && a.cast_src) ld4(vw, a.cast_src, k, vec, cnt);
     } else {
-      ld4(vw, a.cast_src, k, vec, cnt);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) vu[j] = vw[j];
+      for (int j = 0; j < 4; ++j) vu[j] = vw[j] = i.x0[j];
     }
     if (cast_w && tab.W[l]) st_copy<T>(static_cast<T*>(tab.W[l]), e0, r0, dout, din, tab.ldw[l], vw, vec, cnt);
     if (cast_u && tab.U[l]) st_copy<T>(static_cast<T*>(tab.U[l]), e0, r0, dout, din, tab.ldw[l], vu, vec, cnt);
   }
   if (bad && a.status) atomicMax(a.status, DEV_NONFINITE);
-  if (a.partials) {   // one deterministic partial sum per block (scalar log-lr)
-    acc = warp_sum(acc);
-    if ((tid & 31) == 0) red[tid >> 5] = acc;
-    sync();
-    if (tid < 32) {
-      float v = tid < UPD_THREADS / 32 ? red[tid] : 0.f;
-      v = warp_sum(v);
-      if (tid == 0) a.partials[blk] = v;
+  if (a.partials) {   // one deterministic partial sum per tile (scalar log-lr)
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      if (blk + q >= tab.tile0[tab.n]) break;
+      const float w = warp_sum(acc[q]);
+      if ((tid & 31) == 0) red[tid >> 5] = w;
+      sync();
+      if (tid < 32) {
+        float v = tid < UPD_THREADS / 32 ? red[tid] : 0.f;
+        v = warp_sum(v);
+        if (tid == 0) a.partials[blk + q] = v;
+      }
+      sync();   // red may be used again
     }
-    sync();   // red may be used again
   }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(UPD_THREADS) layer_update_kernel(const LayerTable tab,
-                                                                   const LayerUpdArgs a) {
+// The table and the arguments stay in constant memory: indexed by a run-time layer, a by-value
+// copy of them went to each thread's local memory.
+template <typename T, int MODE, bool ADAM, int NQ>
+__global__ void __launch_bounds__(UPD_THREADS) layer_update_kernel(
+    const __grid_constant__ LayerTable tab, const __grid_constant__ LayerUpdArgs a) {
   pdl_entry();
   __shared__ float red[UPD_THREADS / 32];
-  layer_update_block<T>(tab, a, static_cast<int>(blockIdx.x), static_cast<int>(threadIdx.x), red,
-                        [] { __syncthreads(); });
+  layer_update_block<T, MODE, ADAM, NQ>(tab, a, static_cast<int>(blockIdx.x) * NQ,
+                                  static_cast<int>(threadIdx.x), red, [] { __syncthreads(); });
 }
 
 // Reverse-over-reverse, forward layer order: from dzbar (the adjoint of the backward's dz)
@@ -829,7 +890,7 @@ __device__ __forceinline__ void move_op(SmallOp& op, const MovePtr& mv) {
   }
 }
 
-__global__ void __launch_bounds__(SP_THREADS) small_program_kernel(
+__global__ void __launch_bounds__(SP_THREADS, 1) small_program_kernel(
     const __grid_constant__ SmallProgram prog) {
   __shared__ float red[SP_THREADS / 32];
   extern __shared__ __align__(256) char image[];   // the workspace, then the program
@@ -856,9 +917,13 @@ __global__ void __launch_bounds__(SP_THREADS) small_program_kernel(
       }
       case SMALL_UPDATE: {   // a group of UPD_THREADS threads per block of the update
         const LayerUpdArgs& a = *reinterpret_cast<const LayerUpdArgs*>(op.data);
-        for (int b = grp; b < tab.tile0[tab.n]; b += SP_GROUPS)
-          layer_update_block<float>(tab, a, b, tid % UPD_THREADS, red + grp * (UPD_THREADS / 32),
-                                    [&] { asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(UPD_THREADS) : "memory"); });
+        auto tiles = [&](auto mode, auto adam) __attribute__((always_inline)) {
+          for (int b = grp; b < tab.tile0[tab.n]; b += SP_GROUPS)
+            layer_update_block<float, decltype(mode)::value, decltype(adam)::value, 1>(
+                tab, a, b, tid % UPD_THREADS, red + grp * (UPD_THREADS / 32),
+                [&] { asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(UPD_THREADS) : "memory"); });
+        };
+        with_update_mode(a, tiles);
         break;
       }
       case SMALL_COPY: {   // rows x cols floats; a null source writes value
@@ -983,7 +1048,15 @@ void layer_update(const LayerTable& tab, const LayerUpdArgs& args, cudaStream_t 
   if (blocks <= 0) return;
   LayerUpdArgs a = args;
   a.vec_ok = update_vec_ok(a);
-  launch_k(layer_update_kernel<T>, dim3(blocks), dim3(UPD_THREADS), 0, s, tab, a);
+  // A cast has one load a tile, so a block takes four tiles (a Hessian-vector product with 92
+  // million parameters: 2407 us with one, 2365 with four); the other modes have up to
+  // six and lose more to the registers of a second tile (8 x 4096 layers: rollout 6.83 -> 6.98
+  // ms a call with two, adjoint -> 7.28).
+  with_update_mode(a, [&](auto mode, auto adam) {
+    constexpr int MODE = decltype(mode)::value, NQ = MODE == LU_CAST ? 4 : 1;
+    launch_k(layer_update_kernel<T, MODE, decltype(adam)::value, NQ>,
+             dim3((blocks + NQ - 1) / NQ), dim3(UPD_THREADS), 0, s, tab, a);
+  });
 }
 
 template <typename T>
