@@ -14,9 +14,10 @@
 // Roles per CTA (as in the one-tile pair kernel): warp 0 issues the TMA loads of this CTA's
 // 128 rows of A and BN/2 rows of B; warp 1 owns TMEM, and in the even CTA one thread issues
 // tcgen05.mma.cta_group::2 (M = 256) for the pair; epi_warps_p warps drain this CTA's 128
-// accumulator rows, one TMEM lane quadrant and one column share per warp; full 16-column
-// chunks are stored through a 2 KB row-block buffer per warp (8 rows x 64 bytes per warp
-// store, see epilogue16_rows), ragged ones straight from registers.
+// accumulator rows, one TMEM lane quadrant and one column share per warp; the accumulators of
+// full 16-column chunks change to a layout of quads through a 2 KB buffer per warp (8 rows x
+// 64 bytes per warp access, see rows_to_quads) in which everything else is loaded, computed
+// and stored, ragged ones are finished from the row layout.
 //
 // Barriers: full[s] / empty[s] per pipeline stage (full in the even CTA, completed by both
 // CTAs' TMA bytes; empty in both, by the MMA commit multicast); per accumulator set,
