@@ -501,16 +501,7 @@ __device__ __forceinline__ void st_copy(T* W, int64_t e0, int r0, int dout, int 
   }
 }
 
-// Block blk of the update over the whole vector, by UPD_THREADS threads tid (red: one float a
-// warp; sync: their barrier).  Memory traffic bounds it, so a vector that no later operation
-// reads is not written and one that would be zeros is not read: u' where its operand copy
-// serves the products, and the sum of the first learning-rate gradients.  Eight 4096-wide
-// layers, momentum, per-parameter rates, 32 steps: 8.08 -> 8.03 ms a call; 256-512-512-128,
-// 64 steps: 978 -> 957 us.
-// One kernel per mode, so that each has the registers of its own vectors only, and its layer
-// table read from constant memory (a per-thread copy of it in local memory cost more than the
-// search for the layer): the same calls 7.33 -> 6.77 ms and 912 -> 846 us, a 1024-wide one
-// 3.92 -> 3.80 ms.
+// f(mode, adam) of an update as types.
 #pragma nv_exec_check_disable
 template <class F>
 __host__ __device__ __forceinline__ void with_update_mode(const LayerUpdArgs& a, F&& f) {
@@ -523,7 +514,16 @@ __host__ __device__ __forceinline__ void with_update_mode(const LayerUpdArgs& a,
   else f(std::integral_constant<int, LU_CAST>{}, std::false_type{});
 }
 
-// Tiles blk .. blk + NQ - 1, whose loads are all issued before the first result is needed.
+// Tiles blk .. blk + NQ - 1 of the update over the whole vector, by UPD_THREADS threads tid
+// (red: one float a warp; sync: their barrier), whose loads are all issued before the first
+// result is needed.  Memory traffic bounds it, so a vector that no later operation reads is not
+// written and one that would be zeros is not read: u' where its operand copy serves the
+// products, and the sum of the first learning-rate gradients.  Eight 4096-wide layers, momentum,
+// per-parameter rates, 2 steps: 8.08 -> 8.03 ms a call; one 4096 x 4096 layer, 2 steps: 978 ->
+// 957 us.  One kernel per mode, so that each has the registers of its own vectors only, and its
+// layer table read from constant memory (a per-thread copy of it in local memory cost more than
+// the search for the layer): the same calls 7.33 -> 6.77 ms and 912 -> 846 us, a 1024-wide one of
+// 16 steps 3.92 -> 3.80 ms.
 template <typename T, int MODE, bool ADAM, int NQ, class Sync>
 __device__ __forceinline__ void layer_update_block(const LayerTable& tab, const LayerUpdArgs& a,
                                                    int blk, int tid, float* red, Sync sync) {
