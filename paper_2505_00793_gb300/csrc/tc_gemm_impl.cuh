@@ -149,6 +149,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* s
   }
 }
 
+// The same for a whole warp: all its lanes go on, or none.  What follows a wait of the epilogue
+// warps is collective (TMEM loads, warp and CTA barriers), and a limit may expire in one lane
+// while the phase completes for the next.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int* status,
+                                               long long limit_ns) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, status, limit_ns));
+}
+
 // The producer's drain: wait for the last phase issued on every stage (issued = number of K
 // blocks whose loads were issued, in ring order).
 __device__ __forceinline__ void drain_loads(uint64_t* full_bar, int issued, int stages,
@@ -326,6 +334,19 @@ __device__ __forceinline__ uint32_t dsmem_addr(uint32_t local_addr, uint32_t ran
 
 __device__ __forceinline__ void epi_bar() {   // the epilogue warps only
   asm volatile("bar.sync 1, %0;" ::"n"(EPI_THREADS) : "memory");
+}
+// The same barrier; true when `ok` holds in every one of its threads.
+__device__ __forceinline__ bool epi_bar_all(bool ok) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "bar.red.and.pred q, 1, %2, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(r)
+      : "r"(static_cast<uint32_t>(ok)), "n"(EPI_THREADS)
+      : "memory");
+  return r != 0;
 }
 
 // Row-per-thread epilogue for 16 consecutive columns (no split): float32 outputs and the
@@ -1221,9 +1242,11 @@ __global__ void __launch_bounds__(THREADS, 1)
     EpiIn in0;
     if (u_row < rows_per)
       epi_load<MODE>(in0, p, m0 + r_begin + u_row, n0 + u_col, dual);
-    const bool ok = nk > 0 && mbar_wait(&acc_bar, 0, p.status, p.wait_ns);
-    // a peer waits for this CTA's partial sums whether or not the wait gave up
-    if (S > 1 && nk > 0 && !ok) mbar_wait(&acc_bar, 0, p.status, DRAIN_NS);
+    // The limit may expire in one warp and not in the next, and barriers of all of them (and,
+    // under split K, peers that wait for this CTA's partial sums) follow: a warp whose wait
+    // gave up waits for the CTA's own work to drain and goes the same way.
+    const bool ok = nk > 0 && mbar_wait_warp(&acc_bar, 0, p.status, p.wait_ns);
+    if (nk > 0 && !ok) mbar_wait_warp(&acc_bar, 0, p.status, DRAIN_NS);
     // the pipeline buffers are free: warps 0 and 1, which saw the last loads and products
     // complete, release that; these warps have nothing to publish (a releasing arrive took
     // 1,000 clocks)
@@ -1250,22 +1273,20 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
     };
     if (S == 1) {
-      if (ok) {
 #pragma unroll 1
-        for (int cb = 0; cb < BN; cb += CW) {
-          if (cb > 0) epi_bar();   // the previous columns have been read
-          fill(cb);
-          epi_bar();
+      for (int cb = 0; cb < BN; cb += CW) {
+        if (cb > 0) epi_bar();   // the previous columns have been read
+        fill(cb);
+        if (!epi_bar_all(ok)) break;   // in all warps or in none: nothing is stored
 #pragma unroll 1
-          for (int u = e; u < BM * VPR; u += EPI_THREADS) {
-            const int row = u / VPR, col = u % VPR * 4;
-            const int m = m0 + row, n = n0 + cb + col;
-            if (u != e || cb > 0) epi_load<MODE>(in0, p, m, n, dual);
-            const float4 x0 = *reinterpret_cast<const float4*>(tile + ET::at(row, col));
-            float4 x1 = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (dual) x1 = *reinterpret_cast<const float4*>(tile + ET::at(BM + row, col));
-            epi_quad<MODE, ACT>(p, m, n, x0, x1, in0, dual);
-          }
+        for (int u = e; u < BM * VPR; u += EPI_THREADS) {
+          const int row = u / VPR, col = u % VPR * 4;
+          const int m = m0 + row, n = n0 + cb + col;
+          if (u != e || cb > 0) epi_load<MODE>(in0, p, m, n, dual);
+          const float4 x0 = *reinterpret_cast<const float4*>(tile + ET::at(row, col));
+          float4 x1 = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (dual) x1 = *reinterpret_cast<const float4*>(tile + ET::at(BM + row, col));
+          epi_quad<MODE, ACT>(p, m, n, x0, x1, in0, dual);
         }
       }
     } else {
@@ -1290,7 +1311,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
       }
       __syncwarp();
-      mbar_wait(&recv_bar, 0, p.status, DRAIN_NS);
+      mbar_wait_warp(&recv_bar, 0, p.status, DRAIN_NS);
       // the peers' copies out of their tiles to this CTA are complete (nothing is published:
       // a releasing arrive took 1,000 clocks)
       cluster_arrive_relaxed();
