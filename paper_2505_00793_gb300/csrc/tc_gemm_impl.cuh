@@ -1643,7 +1643,7 @@ __global__ void __launch_bounds__(THREADS2, 1)
     const uint32_t lane_off = static_cast<uint32_t>(q * 32) << 16;
     constexpr int CG = BN / EPI_GROUPS2;
     const int c_begin = ((warp - 2) >> 2) * CG, c_end = c_begin + CG;
-    const bool ok = mbar_wait(&acc_bar, 0, p.status, p.wait_ns);
+    const bool ok = mbar_wait_warp(&acc_bar, 0, p.status, p.wait_ns);
     tc_fence_after();
     if (ok) {
       if (p.tma_store) {

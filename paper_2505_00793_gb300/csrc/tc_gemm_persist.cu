@@ -377,7 +377,11 @@ __global__ void __launch_bounds__(threads_p<MODE>(), 1)
     for (int t = pair; t < pp.ntiles; t += npairs, ++j) {
       const int set = pp.nsets == 2 ? (j & 1) : 0;
       const int use = pp.nsets == 2 ? (j >> 1) : j;
-      if (!pwait<false>(&acc_full[set], use & 1, p.status, abort, p.wait_ns)) break;
+      // all lanes of the warp go on or none: the TMEM loads and the row buffer's warp barriers
+      // that follow are collective
+      if (!__all_sync(0xffffffffu,
+                      pwait<false>(&acc_full[set], use & 1, p.status, abort, p.wait_ns)))
+        break;
       tc_fence_after();
       int bz, mp, tn;
       coords(t, bz, mp, tn);

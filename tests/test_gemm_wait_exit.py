@@ -1,5 +1,5 @@
 """How the tcgen05 GEMMs' epilogue warps leave a wait whose limit expires
-(csrc/tc_gemm_impl.cuh).
+(csrc/tc_gemm_impl.cuh, csrc/tc_gemm_persist.cu).
 
 On the CPU: the one-SM epilogue's waits and barriers as coroutines, a lane each, in which any set
 of lanes may see the limit expire while the accumulator arrives for the others.  Every schedule
@@ -113,25 +113,33 @@ def test_model_catches_planted_mistakes(rule):
     assert stuck > 20
 
 
-@pytest.mark.parametrize("name", ["tc_gemm_impl.cuh"])
-def test_limited_waits_are_voted(name):
+def _source(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//[^\n]*", "", f.read())
+
+
+def test_limited_waits_are_voted():
     """A wait of the epilogue warps on the accumulator returns one answer a warp; the one-SM
     kernel's barriers of all epilogue warps stand under no condition on it."""
-    with open(os.path.join(CSRC, name)) as f:
-        src = re.sub(r"//[^\n]*", "", f.read())
-    body = src[src.index("tc_dual_gemm_kernel("):src.index("typedef CUresult")]
-    waits = re.findall(r"(\w+)\(&(acc_bar|recv_bar), 0, p\.status, (p\.wait_ns|DRAIN_NS)\)", body)
-    epilogue = waits[1:]   # the first one is the MMA issuer's, a single thread
-    assert len(epilogue) == 3 and {w for w, _, _ in epilogue} == {"mbar_wait_warp"}
-    assert not re.search(r"if \(ok\b", body)
+    src = _source("tc_gemm_impl.cuh")
+    one = src[src.index("tc_dual_gemm_kernel("):src.index("typedef CUresult")]
+    pair = src[src.index("tc2_dual_gemm_kernel("):src.index("launch_cfg2(")]
+    for body, n in ((one, 3), (pair, 1)):
+        waits = re.findall(r"(\w+)\(&(acc_bar|recv_bar), 0, p\.status, (p\.wait_ns|DRAIN_NS)\)", body)
+        epilogue = waits[1:]   # the first one is the MMA issuer's, a single thread
+        assert len(epilogue) == n and {w for w, _, _ in epilogue} == {"mbar_wait_warp"}
+    assert not re.search(r"if \(ok\b", one)
+    src = _source("tc_gemm_persist.cu")
+    waits = re.findall(r"(\S+)\s*pwait<false>\(&acc_full", src)
+    assert waits == ["(!__all_sync(0xffffffffu,"]
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("kernel", ["one_sm"])
+@pytest.mark.parametrize("kernel", ["one_sm", "pair", "persistent"])
 @pytest.mark.parametrize("limit_us", [0, 1, 3, 6, 12, 40])
 def test_limits_around_a_product(kernel, limit_us):
     torch, native = need_gpu()
-    # unsplit and split products
+    # unsplit and split products of one-SM tiles; more than 128 rows for the pair tiles
     w = synth.Workload("limit", [128, 256, 512, 136, 10], "gelu", "ce", "bf16", B=160, T=2,
                        B_outer=96, alpha=0.05)
     d = native.to_device_inputs(w, synth.make_inputs(w))
@@ -146,7 +154,8 @@ def test_limits_around_a_product(kernel, limit_us):
 
     try:
         mf.set_option(native.MF_OPT_CUDA_GRAPHS, 0)
-        mf.set_option(native.MF_OPT_GEMM_2SM, 0)
+        mf.set_option(native.MF_OPT_GEMM_2SM, 0 if kernel == "one_sm" else 2)
+        mf.set_option(native.MF_OPT_GEMM_PERSISTENT, int(kernel == "persistent"))
         ref = call()
         mf.set_option(native.MF_OPT_WAIT_LIMIT_US, limit_us)
         for _ in range(4):
@@ -161,5 +170,6 @@ def test_limits_around_a_product(kernel, limit_us):
         assert all(np.array_equal(a, b) for a, b in zip(call(), ref))
     finally:
         mf.set_option(native.MF_OPT_WAIT_LIMIT_US, 2000000)
+        mf.set_option(native.MF_OPT_GEMM_PERSISTENT, 2)
         mf.set_option(native.MF_OPT_GEMM_2SM, 1)
         mf.close()
