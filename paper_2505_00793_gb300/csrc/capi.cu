@@ -693,7 +693,7 @@ struct Exec {
         g.bias1 = h->md.has_bias ? u + h->boff[l] : nullptr;
       }
       if (l + 1 < h->L) {
-        if (keep_d2) { g.C1 = at<float>(p.o_Zd[l]); g.ldc1 = dout; }
+        if (keep_d2) { g.keep_d2 = true; g.C1 = at<float>(p.o_Zd[l]); g.ldc1 = dout; }
         g.epi.mode = mf::EPI_ACT_FWD;
         g.epi.act = h->md.act;
         g.epi.A = at<T>(p.o_A[l + 1]);

@@ -434,7 +434,7 @@ struct DecExec {
                          ld8(F), dual);
         g.b_mn = true;
         g.C0 = at<float>(p.z1[l]); g.ldc0 = F;
-        g.C1 = at<float>(p.z1d[l]); g.ldc1 = F;
+        g.C1 = dual ? at<float>(p.z1d[l]) : nullptr; g.ldc1 = F;
         g.epi.mode = mf::EPI_ACT_FWD;
         g.epi.act = mf::ACT_GELU;
         g.epi.A = at<T>(p.a1[l]);

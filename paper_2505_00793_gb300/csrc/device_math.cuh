@@ -49,8 +49,9 @@ __device__ __forceinline__ void act_eval(int act, float z, float& f, float& d1, 
 //  EPI_ACT_FWD: z = acc0 + bias0, z' = acc1 + bias1 ->
 //               a = phi(z), a' = phi'(z) z'  -> A, Ad (row-major), and what the backward pass
 //               needs of z, in place of z itself: phi'(z) -> C0 and, where C1 is given,
-//               phi''(z) z' (dual) or phi''(z) (primal) -> C1, float32.  The activation is
-//               evaluated once per element and pass instead of again in the backward.
+//               phi''(z) z' (dual) or phi''(z) (primal, GemmArgs::keep_d2) -> C1, float32.  The
+//               activation is evaluated once per element and pass instead of again in the
+//               backward.
 //  EPI_ACT_BWD: da = acc0, da' = acc1, the stored derivatives read from Z, Zd ->
 //               dz = Z da, dz' = Zd da + Z da'  -> A, Ad.
 struct EpiOut {

@@ -89,13 +89,14 @@ struct GemmArgs {
   // Operand layouts: K-major (default, X[row][k] at row * ld + k) or MN-major
   // (X[row][k] at k * ld + row), for A0/A1 and for B0/B1.
   bool a_mn = false, b_mn = false;
+  bool keep_d2 = false;    // primal EPI_ACT_FWD: phi''(z) goes to C1
   int* status = nullptr;   // device status word (timeouts), may be null
 };
 
 // Whether the epilogue writes C1: a second accumulator, or the second derivative that a
-// primal forward epilogue leaves there.
+// primal forward epilogue leaves there on request.
 inline bool writes_c1(const GemmArgs& a) {
-  return (a.terms & (T_C1_A1B0 | T_C1_A0B1)) || a.epi.mode == EPI_ACT_FWD;
+  return (a.terms & (T_C1_A1B0 | T_C1_A0B1)) || (a.epi.mode == EPI_ACT_FWD && a.keep_d2);
 }
 
 // tcgen05 bf16 GEMM (tc_gemm.cu).  Returns cudaSuccess or the launch error; sets *why on a
