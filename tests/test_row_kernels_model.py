@@ -1,16 +1,18 @@
 """Index arithmetic and summation order of the decoder's token-ordering and embedding-gradient
 kernels (csrc/decoder_kernels.cu), restated on the CPU.
 
-- scan_kernel: thread t of 1024 owns counts [t per, (t + 1) per); run totals are scanned
-  within warps by shuffles, then over the 32 warp totals; the thread writes its run's
-  exclusive starts, and start[V] is the total.  Must equal the exclusive prefix sum.
+- scan_kernel: a pass takes 4096 counts, four consecutive ones for each of 1024 threads (zeros
+  past the last); their sums are scanned within warps by shuffles, every warp scans the 32
+  warp totals of the pass (in one of two alternating slots), and the block carries the running
+  total to the next pass; start[V] is the last carry.  Must equal the exclusive prefix sum.
 - token_order_kernel: ids are dealt to G blocks with a stride; each id's scattered positions
   (any order) are ranked: segments of up to 32 by counting smaller positions in a warp,
   longer ones through a bitmap of positions (rank = set bits below the position, with the
   words' bit counts prefix-summed by 256 threads) when the batch has at most 65536 tokens.
   Must equal a stable sort of the token ids.
-- rmsnorm_bwd_warp_kernel + gain_grad_final_kernel: every (row, column) of the gain gradient is
-  added into exactly one partial row, and every partial row read once by the final sums.
+- rmsnorm_bwd_warp_kernel, rmsnorm_bwd_block_kernel + gain_grad_final_kernel: every (row, column)
+  of the gain gradient is added into exactly one partial row, and every partial row read once by
+  the final sums.
 - embed_bwd_kernel: a segment of up to 8 rows is summed by one warp in row order from zero; a
   longer one by eight warps over contiguous parts, the parts added in warp order.  For up to
   8 rows both give the same float32 bits."""
@@ -24,24 +26,29 @@ SCAN_THREADS = 1024
 
 def scan_model(count):
     V = len(count)
-    per = -(-V // SCAN_THREADS)
-    runs = [int(np.sum(count[t * per:min(V, t * per + per)], dtype=np.int64))
-            for t in range(SCAN_THREADS)]
-    inc = []
-    for w in range(SCAN_THREADS // 32):
-        acc = 0
-        for lane in range(32):
-            acc += runs[w * 32 + lane]
-            inc.append(acc)
-    wtot = np.cumsum([inc[w * 32 + 31] for w in range(SCAN_THREADS // 32)]).tolist()
-    start = [0] * (V + 1)
-    for t in range(SCAN_THREADS):
-        w = t // 32
-        acc = inc[t] - runs[t] + (wtot[w - 1] if w > 0 else 0)
-        for i in range(t * per, min(V, t * per + per)):
-            start[i] = acc
-            acc += int(count[i])
-    start[V] = wtot[-1]
+    start = [None] * (V + 1)
+    carry, wtot, p = 0, [[None] * 32, [None] * 32], 0
+    for c0 in range(0, V, 4 * SCAN_THREADS):
+        quads = [[int(count[i]) if i < V else 0 for i in range(c0 + 4 * t, c0 + 4 * t + 4)]
+                 for t in range(SCAN_THREADS)]
+        run = [sum(q) for q in quads]
+        inc = []
+        for t in range(SCAN_THREADS):
+            inc.append(run[t] + (inc[-1] if t % 32 else 0))
+            if t % 32 == 31:
+                wtot[p][t // 32] = inc[-1]
+        tot = np.cumsum(wtot[p]).tolist()
+        for t in range(SCAN_THREADS):
+            acc = carry + inc[t] - run[t] + (tot[t // 32 - 1] if t >= 32 else 0)
+            for k in range(4):
+                i = c0 + 4 * t + k
+                if i < V:
+                    assert start[i] is None
+                    start[i] = acc
+                acc += quads[t][k]
+        carry += tot[31]
+        p ^= 1
+    start[V] = carry
     return start
 
 
@@ -77,7 +84,7 @@ def order_model(V, N, start, tmp, G, bitmap_tokens=32 * 2048):
     return order
 
 
-@pytest.mark.parametrize("V", [1, 2, 7, 1024, 1025, 32768, 40000])
+@pytest.mark.parametrize("V", [1, 2, 7, 1024, 1025, 4095, 4096, 4097, 32768, 40000])
 def test_scan_is_exclusive_prefix_sum(V):
     rng = np.random.default_rng(V)
     count = rng.integers(0, 9, V)
@@ -168,3 +175,24 @@ def test_gain_partials_cover_every_row_and_column_once(N, d):
                 for c in range(y, nblk, 32):
                     read[c, j] += 1
     assert (read == 1).all()
+
+
+@pytest.mark.parametrize("N,d", [(2048, 1024), (13, 260), (9, 1028), (64, 1000), (250, 2048)])
+def test_block_kernel_gain_partials(N, d):
+    """The block kernel (256 < d <= 2048): VPT column groups a thread (one up to 1024 columns,
+    two above), 4 blockDim apart, over the rows 8b .. min(N, 8b + 8) of block b; the gain's
+    partial row b takes every column once."""
+    vpt = 1 if d <= 1024 else 2
+    threads = -(-d // (128 * vpt)) * 32
+    assert threads <= 256 and vpt * 4 * threads >= d
+    nblk = (N + 7) // 8
+    contrib = np.zeros((N, d), np.int32)
+    written = np.zeros((nblk, d), np.int32)
+    for b in range(nblk):
+        for t in range(threads):
+            for k in range(vpt):
+                c = 4 * (t + k * threads)
+                if c < d:
+                    written[b, c:c + 4] += 1
+                    contrib[8 * b:min(N, 8 * b + 8), c:c + 4] += 1
+    assert (written == 1).all() and (contrib == 1).all()
