@@ -1992,6 +1992,8 @@ mf_status mf_sync(mf_handle h) {
     cudaMemset(h->d_status, 0, sizeof(int));
     if (v == mf::DEV_TIMEOUT) return fail(h, MF_ERR_TIMEOUT, "a device-side wait ran out of time");
     if (v == mf::DEV_NONFINITE) return fail(h, MF_ERR_NONFINITE, "non-finite value in the adjoint or the parameters");
+    if (v == mf::DEV_SMEM_BASE)
+      return fail(h, MF_ERR_CUDA, "a kernel's dynamic shared memory is not 1024-byte aligned");
     if (v == 1) return fail(h, MF_ERR_INVALID_ARG, "a class label is out of range");
     return fail(h, MF_ERR_CUDA, "device status " + std::to_string(v));
   }

@@ -598,6 +598,8 @@ struct KvCfg {
   static constexpr int SLACK = DUAL ? 0 : 1024;
   static constexpr int SMEM =
       NRES * ROWS128_B + STAGES * STAGE_B + NOP * OPND_B + 2 * STAT_B + SLACK;
+  // 227 KB a CTA, of which the barriers and flags (static) take the first 1024 bytes
+  static_assert(SMEM + 1024 <= 227 * 1024, "the key-tile kernel's shared memory fits a CTA");
   static constexpr int CTAS = DUAL ? 1 : 2;
   static constexpr uint32_t TMEM_COLS = DUAL ? 512 : 256;
   static constexpr uint32_t C_S = 0, C_SD = 64, C_DP = DUAL ? 128 : 64, C_DPD = 192;
@@ -738,7 +740,7 @@ __global__ void __launch_bounds__(KvCfg<DUAL>::THREADS, KvCfg<DUAL>::CTAS)
   uint8_t* sOp = sSt + C::STAGES * C::STAGE_B;           // P^T, dS^T, P'^T, dS'^T
   float* sStat = reinterpret_cast<float*>(sOp + C::NOP * OPND_B);   // two tiles' statistics
   if (C::SLACK == 0 && smem != smem_raw) {   // the whole grid alike, before any barrier
-    if (threadIdx.x == 0 && p.status) atomicMax(p.status, DEV_TIMEOUT);
+    if (threadIdx.x == 0 && p.status) atomicMax(p.status, DEV_SMEM_BASE);
     return;
   }
   // grid (heads, key tiles): heads fastest, and key tile 0 meets the most query tiles

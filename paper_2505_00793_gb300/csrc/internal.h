@@ -40,11 +40,12 @@ struct PerDeviceOnce {
   }
 };
 
-// Device status word values (also the mf_status codes they map to).
+// Device status word values (up to 6 the mf_status codes they map to).
 // Kernels raise the word with atomicMax, so the most severe condition of a call survives:
-// a timed-out wait (whose skipped work leaves garbage behind) over a non-finite value over
+// a kernel that found its shared memory at an address it cannot use and did nothing over a
+// timed-out wait (whose skipped work leaves garbage behind) over a non-finite value over
 // an out-of-range label (1).
-enum : int { DEV_OK = 0, DEV_NONFINITE = 5, DEV_TIMEOUT = 6 };
+enum : int { DEV_OK = 0, DEV_NONFINITE = 5, DEV_TIMEOUT = 6, DEV_SMEM_BASE = 7 };
 
 // GEMM product terms (same bit meaning as mf_dual_gemm_bf16's `terms`).
 enum : unsigned {
