@@ -540,6 +540,7 @@ struct Exec {
     if (st != MF_OK) return;
     const cudaStream_t s = on ? on : this->s;
     g.status = h->d_status;
+    if (!mf::writes_c1(g)) g.C1 = nullptr;   // what the launchers do, for the program too
     if (record(mf::SMALL_GEMM, g)) return;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     unsigned ev_flags = cudaEventRecordDefault;
@@ -733,7 +734,10 @@ struct Exec {
       head(rows, dual, a, fwd_theta, fwd_u);
       return;
     }
-    if (record(mf::SMALL_LOSS, a)) return;
+    seed(a);
+  }
+  void seed(const mf::LossArgs& a) {
+    if (!mf::loss_ready(a) || record(mf::SMALL_LOSS, a)) return;
     mf::loss_seed<T>(a, s);
     launched();
   }
@@ -918,10 +922,7 @@ struct Exec {
           a.tape = at<float>(p.o_CH);
           a.ror = 2;
         }
-        if (!record(mf::SMALL_LOSS, a)) {
-          mf::loss_seed<T>(a, s);
-          launched();
-        }
+        seed(a);
       }
     }
     // adjoint of the forward pass, layers L-1..0

@@ -159,6 +159,10 @@ struct LossArgs {
   float* tape = nullptr;
   int ror = 0;
 };
+// Whether there is a loss to compute: rows, logits and the targets that its kind reads.
+inline bool loss_ready(const LossArgs& a) {
+  return a.rows > 0 && a.F && (a.loss == 1 ? a.Yi != nullptr : a.Yf != nullptr);
+}
 template <typename T>
 void loss_seed(const LossArgs& a, cudaStream_t s);
 

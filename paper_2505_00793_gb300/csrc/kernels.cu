@@ -992,8 +992,7 @@ void fill_cols(const ColFill& f, int rows, cudaStream_t s) {
 
 template <typename T>
 void loss_seed(const LossArgs& a, cudaStream_t s) {
-  if (a.rows <= 0) return;
-  if ((a.loss == 1 && !a.Yi) || (a.loss != 1 && !a.Yf) || !a.F) return;   // no targets: nothing read
+  if (!loss_ready(a)) return;
   // sixteen-byte access where every row is a multiple of it
   auto al = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
   const bool vec = !(a.cols & 3) && !(a.ldo & 3) && al(a.F) && al(a.Fd) && al(a.Yf) && al(a.dF) && al(a.dFd);
