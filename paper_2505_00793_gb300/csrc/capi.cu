@@ -833,7 +833,6 @@ struct Exec {
       d.B1 = at<T>(p.o_Ub[l]); d.ldb1 = ld8(dout);
       d.terms = dual ? (mf::T_C0_A0B0 | mf::T_C1_A1B0 | mf::T_C1_A0B1) : mf::T_C0_A0B0;
       d.epi.mode = mf::EPI_ACT_BWD;
-      d.epi.act = h->md.act;
       d.epi.Z = at<float>(p.o_Z[l - 1]);
       d.epi.Zd = dual ? at<float>(p.o_Zd[l - 1]) : nullptr;
       d.epi.ldz = din;

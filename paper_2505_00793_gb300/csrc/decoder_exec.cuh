@@ -647,7 +647,6 @@ struct DecExec {
       {
         GemmArgs g = lin(N, F, d, at<T>(p.dy), at<T>(p.dyd), d, W(Ly.W2[l]), Uw(Ly.W2[l]), ld8(d), dual);
         g.epi.mode = mf::EPI_ACT_BWD;
-        g.epi.act = mf::ACT_GELU;
         g.epi.Z = at<float>(p.z1[l]);
         g.epi.Zd = dual ? at<float>(p.z1d[l]) : nullptr;
         g.epi.ldz = F;

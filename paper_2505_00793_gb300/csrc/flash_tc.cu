@@ -583,7 +583,7 @@ constexpr int OPND_B = 128 * 64 * 2;           // 16 KB: [128][64] bf16 A operan
 
 template <bool DUAL>
 struct KvCfg {
-  static constexpr int EW = DUAL ? 8 : 8;       // elementwise warps
+  static constexpr int EW = 8;                 // elementwise warps
   static constexpr int THREADS = 64 + 32 * EW;
   static constexpr int NRES = DUAL ? 4 : 2;    // K, V (K', V'): 128 rows each
   static constexpr int NT = DUAL ? 4 : 2;      // Q, (Q',) dO (, dO') per query tile: 64 rows
@@ -609,7 +609,7 @@ struct KvCfg {
 
 template <bool DUAL>
 struct QCfg {
-  static constexpr int EW = DUAL ? 8 : 8;
+  static constexpr int EW = 8;                 // elementwise warps
   static constexpr int THREADS = 64 + 32 * EW;
   static constexpr int NRES = DUAL ? 4 : 2;    // Q, dO (Q', dO'): 128 rows each
   static constexpr int NT = DUAL ? 4 : 2;      // K, (K',) V (, V') per key tile: 64 rows
@@ -1401,11 +1401,7 @@ bool flash_tc_bwd_supported(const FlashArgs& a, bool dual) {
                  (reinterpret_cast<uintptr_t>(a.dqkv) & 15) ||
                  (dual && (!a.dqkvd || (reinterpret_cast<uintptr_t>(a.dqkvd) & 15)))))
     return false;
-  // the row statistics stream into shared memory by bulk copies of 64 floats
-  const void* stats[4] = {a.lse, a.D, a.rbar, a.Dd};
-  for (int i = 0; i < (dual ? 4 : 2); ++i)
-    if (!stats[i] || (reinterpret_cast<uintptr_t>(stats[i]) & 15)) return false;
-  return true;
+  return a.lse && a.D && (!dual || (a.rbar && a.Dd));   // row statistics, read a float at a time
 }
 
 cudaError_t flash_tc_bwd(const FlashArgs& a, bool dual, cudaStream_t s) {

@@ -84,8 +84,7 @@ struct GemmArgs {
   EpiParams epi;
   int batch = 1;           // independent GEMMs of the same shape (attention heads)
   int64_t bsA0 = 0, bsA1 = 0, bsB0 = 0, bsB1 = 0, bsC0 = 0, bsC1 = 0;   // batch strides (elements)
-  int split_k = 0;         // 0 = choose automatically, else 1/2/4/8 (tensor-core path)
-  int bn = 0, ka = 0;      // tile width / K atoms per stage; 0 = choose automatically
+  int bn = 0;              // tile width; 0 = choose automatically
   int pair = 0;            // 2-SM tiles (tensor-core path): 0 automatic, 1 always, -1 never
   // Operand layouts: K-major (default, X[row][k] at row * ld + k) or MN-major
   // (X[row][k] at k * ld + row), for A0/A1 and for B0/B1.

@@ -73,7 +73,7 @@ cudaError_t tc_gemm(const GemmArgs& a, cudaStream_t s, const char** why) {
   }
   int bn = a.bn, pair = 0;
   const int nbatch = a.batch < 1 ? 1 : a.batch;
-  if (a.pair >= 0 && a.split_k <= 1 && a.M > 128 && (bn == 0 || bn == 128 || bn == 256)) {
+  if (a.pair >= 0 && a.M > 128 && (bn == 0 || bn == 128 || bn == 256)) {
     // 2-SM tiles (256 rows per CTA pair) when the pair grid fills the GPU
     const int pairs_m = ((a.M + 255) / 256) * nbatch;
     if (a.pair == 1 || g_pair_mode == 2) {

@@ -999,19 +999,15 @@ __device__ __forceinline__ void mma_dispatch(const MmaLoop& L, unsigned terms, i
 }
 
 // ---- epilogue of the one-SM kernel ------------------------------------------------------
-// Small tiles are bound by the latency of a chain of steps, not by any unit: of the 21 k
-// clocks of a 256 x 1024 x 1024 dual GELU layer (K split four ways), 6 k were loads and MMAs,
-// 10 k the exchange (sixteen-byte remote stores between two cluster barriers, then a pass
-// that added the slabs) and 4 k an epilogue of one column and eight rows per thread.  The
-// tile now crosses shared memory once, bulk copies move contiguous slabs to their owners and
-// complete a barrier there, the sum is fused with the epilogue at four columns of one row per
-// thread, and the stored inputs load during the main loop.  Wide MLP meta-gradient (462 such
-// GEMMs) 5.33 -> 4.31 ms, ragged reverse-over-reverse step 240 -> 202 us, transformer with
-// 96-wide heads 1.96 -> 1.75 ms.  Of the 15,000 clocks of a 256 x 1024 x 1024 dual product split
-// four ways, the main loop takes 5,400 (L2 reads) and the exchange 2,700; the accumulator
-// blocks are loaded together, the partial sums of a quad too, and only warps with something
-// to publish release the cluster barriers (9.25 -> 8.5 us in a chain of such products, with
-// stored derivatives 8.6 -> 7.8; the wide meta-gradient 4.22 -> 3.95 ms).
+// Small tiles are bound by the latency of a chain of steps, not by any unit.  The tile crosses
+// shared memory once, bulk copies move contiguous slabs to their owners and complete a barrier
+// there, the sum is fused with the epilogue at four columns of one row per thread, the
+// accumulator blocks are loaded together and the partial sums of a quad too, the stored inputs
+// load during the main loop, and only warps with something to publish release the cluster
+// barriers.  A 256 x 1024 x 1024 dual layer, K split four ways: 21,000 -> 15,000 clocks against
+// remote stores between two cluster barriers, a pass that added the slabs and one column per
+// thread; 5,400 of them are the main loop (L2 reads), 2,700 the exchange.  8.5 us a launch in a
+// chain of such products, 7.8 with stored derivatives.
 __device__ __forceinline__ void cluster_arrive() {
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
@@ -1344,8 +1340,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
       };
       if (S == 2) finish(std::integral_constant<int, 2>{});
-      else if (S == 4) finish(std::integral_constant<int, 4>{});
-      else finish(std::integral_constant<int, 8>{});
+      else finish(std::integral_constant<int, 4>{});
       __syncwarp();
       cluster_wait();
     }
@@ -1423,8 +1418,8 @@ bool make_op_map(CUtensorMap* m, const void* ptr, int K, int rows, int ld, int b
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
-// Split of K across a cluster: double S while the grid stays within ~1.2 waves of 152 SMs
-// and every split keeps at least two K stages.
+// Split of K across a cluster (1, 2 or 4): double S while the grid stays within ~1.2 waves of
+// 152 SMs and every split keeps at least two K stages.
 int choose_split(int tiles, int nkb) {
   int S = 1;
   while (S < 4 && tiles * S * 2 <= 184 && (nkb + 2 * S - 1) / (2 * S) >= 2) S *= 2;
@@ -1464,11 +1459,7 @@ cudaError_t launch_cfg(const GemmArgs& a, cudaStream_t s, const char** why) {
 
   const int tiles_n = (a.N + BN - 1) / BN, tiles_m = (a.M + BM - 1) / BM;
   const int nkb = (a.K + BK * KA - 1) / (BK * KA);
-  int S = a.split_k > 0 ? a.split_k
-                        : (BN > 128 ? 1 : choose_split(tiles_n * tiles_m * (a.batch < 1 ? 1 : a.batch), nkb));
-  if (S != 1 && S != 2 && S != 4 && S != 8) { *why = "split_k must be 1, 2, 4 or 8"; return cudaErrorInvalidValue; }
-  if (BN > 128) S = 1;
-  if (S > nkb) S = 1;
+  int S = BN > 128 ? 1 : choose_split(tiles_n * tiles_m * (a.batch < 1 ? 1 : a.batch), nkb);
 
   CUtensorMap mA0, mA1, mB0, mB1;
   memset(&mA0, 0, sizeof(mA0)); memset(&mA1, 0, sizeof(mA1));
@@ -1536,15 +1527,6 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
-}
-
-__device__ __forceinline__ void tma_load_3d_pair(void* dst, const CUtensorMap* map,
-                                                 uint32_t bar_cluster, int x, int y, int z) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar_cluster)
-      : "memory");
 }
 
 template <int BN, int MODE, int ACT>
