@@ -290,7 +290,11 @@ mf_status mf_replay_gemms(mf_handle h, int reps, void* stream, double* ms, uint6
  * Setting it drops the handle's captured graphs.
  * MF_OPT_CONCURRENT (default 1): in each backward layer the weight product and the data
  * product run on two streams (parallel branches of a captured graph); 0 runs them in
- * sequence on the call's stream.
+ * sequence on the call's stream.  A float32 MLP with a squared or softmax-CE loss, at most 2048
+ * parameters, a largest layer of at most 20480 multiply-adds and at most 160 KB of workspace
+ * runs as one kernel of one block (several, for calls of more than 96 operations) unless
+ * MF_OPT_FUSED_HEAD takes its output layer; this option and MF_OPT_LAYER_UPDATES have no
+ * effect on it.
  * MF_OPT_GEMM_2SM (process-wide): 1 (default) computes a bf16 GEMM with 256-row tiles on
  * CTA pairs (tcgen05 cta_group::2) when its grid of pairs fills the GPU, 0 never, 2 for
  * every GEMM with more than 128 rows (for tests).  Results are identical up to the

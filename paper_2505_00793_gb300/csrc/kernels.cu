@@ -516,14 +516,13 @@ __host__ __device__ __forceinline__ void with_update_mode(const LayerUpdArgs& a,
 
 // Tiles blk .. blk + NQ - 1 of the update over the whole vector, by UPD_THREADS threads tid
 // (red: one float a warp; sync: their barrier), whose loads are all issued before the first
-// result is needed.  Memory traffic bounds it, so a vector that no later operation reads is not
-// written and one that would be zeros is not read: u' where its operand copy serves the
-// products, and the sum of the first learning-rate gradients.  Eight 4096-wide layers, momentum,
-// per-parameter rates, 2 steps: 8.08 -> 8.03 ms a call; one 4096 x 4096 layer, 2 steps: 978 ->
-// 957 us.  One kernel per mode, so that each has the registers of its own vectors only, and its
-// layer table read from constant memory (a per-thread copy of it in local memory cost more than
-// the search for the layer): the same calls 7.33 -> 6.77 ms and 912 -> 846 us, a 1024-wide one of
-// 16 steps 3.92 -> 3.80 ms.
+// result is needed.  Memory traffic bounds it (about 85% of the copy bandwidth on vectors of
+// 537 MB), so a vector that no later operation reads is not written and one that would be zeros
+// is not read: u' where its operand copy serves the products, and the sum of the first
+// learning-rate gradients.  One kernel per mode, so that each has the registers of its own
+// vectors only, and its layer table read from constant memory (a per-thread copy of it in local
+// memory cost more than the search for the layer): against one kernel for all modes, a call of
+// 2 steps on eight 4096-wide layers with momentum and per-parameter rates 7.33 -> 6.80 ms.
 template <typename T, int MODE, bool ADAM, int NQ, class Sync>
 __device__ __forceinline__ void layer_update_block(const LayerTable& tab, const LayerUpdArgs& a,
                                                    int blk, int tid, float* red, Sync sync) {
